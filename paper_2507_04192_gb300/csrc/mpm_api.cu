@@ -192,7 +192,7 @@ void free_particles(mpm_ctx *c)
     dfree(d.S); dfree(d.S2);
     dfree(d.id); dfree(d.id2); dfree(d.sim); dfree(d.sim2);
     dfree(d.keys[0]); dfree(d.keys[1]); dfree(d.vals[0]); dfree(d.vals[1]);
-    dfree(d.hist); dfree(d.tiles); dfree(d.perm); dfree(d.posmap); dfree(d.cell_off); dfree(d.staging);
+    dfree(d.hist); dfree(d.tiles); dfree(d.items); dfree(d.perm); dfree(d.posmap); dfree(d.cell_off); dfree(d.staging);
     c->hp.n = 0;
 }
 
@@ -422,7 +422,10 @@ int load_particles(mpm_ctx *c, int64_t n, const double *x, const double *v, doub
     if (rc == MPM_OK) rc = dalloc(c, &ds.vals[0], n, "values");
     if (rc == MPM_OK) rc = dalloc(c, &ds.vals[1], n, "values");
     if (rc == MPM_OK) rc = dalloc(c, &ds.hist, (size_t)kRadixBins * nblk + kScanSegments, "histogram");
-    if (rc == MPM_OK) rc = dalloc(c, &ds.tiles, 2 * ds.max_tiles, "tile list");     // key order + G2P order
+    if (rc == MPM_OK) rc = dalloc(c, &ds.tiles, ds.max_tiles, "tile list");
+    ds.item_q = g2p_item_size(n, ds.num_sms, c->grid.precision == MPM_FP64);
+    ds.max_items = 2 * ds.max_tiles + (n + 2 * kPB * ds.max_tiles) / ds.item_q + 1;   // ceil per tile, and its cut ends
+    if (rc == MPM_OK) rc = dalloc(c, &ds.items, ds.max_items, "work items");
     if (rc == MPM_OK) rc = dalloc(c, &ds.perm, n, "permutation");
     if (rc == MPM_OK) rc = dalloc(c, &ds.posmap, n, "position map");
     if (rc == MPM_OK) rc = dalloc(c, &ds.cell_off, (size_t)ds.max_tiles * (TN + 1), "cell offsets");

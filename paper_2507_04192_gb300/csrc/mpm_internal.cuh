@@ -133,14 +133,17 @@ struct DevState {
     int32_t *vals[2];
     uint32_t *hist;               // kRadixBins x n_sort_blocks
     int32_t *tile_start, *tile_end;   // per tile (batch x tiles_per_sim)
-    int4 *tiles;                  // compact non-empty tiles: (tile key, start, count, 0) in key order,
-                                  // then (at + max_tiles) the same tiles largest first (G2P order)
+    int4 *tiles;                  // compact non-empty tiles: (tile key, start, count, index) in key order
     int64_t max_tiles;
+    int4 *items;                  // G2P work items: runs of a tile's particles, largest first (same fields)
+    int64_t max_items;
+    int32_t item_q;               // particles per item, at most about (g2p_item_size)
     int32_t *perm;                // gather permutation of the last sort
     int32_t *posmap;              // per particle in (cell, rank) order: its slot relative to the tile start
     int32_t *cell_off;            // per compact tile: TN + 1 exclusive prefix sums of the cell counts
     int32_t *counters;            // [1] n_active_tiles, [2] P2G tile cursor, [3] G2P tile cursor,
-                                  // [4] length of the touched node-tile list
+                                  // [4] length of the touched node-tile list, [5] the adjoint scatter's
+                                  // cursor, [6] number of G2P items
     void *A, *V;                  // grid accumulators and velocities, R4 per node
     uint32_t *flags;              // per node tile: touched since the last grid update
     int32_t *node_list;           // the touched node tiles, in the order P2G touched them
@@ -159,6 +162,20 @@ struct DevState {
     int n_seg[kMaxWalls][2];
     int key_bits;
 };
+
+// Particles per G2P work item, in whole 256-particle rounds of a block: about four
+// items per SM, so that the last ones finish together; at least one round (small
+// problems spread over all SMs) and at most a full 3D tile in single precision, as
+// smaller items cost more window loads than they balance (G2P at 512 / 1024 / 2048
+// / 4096 particles per item: 72.7 / 63.1 / 58.8 / 66.6 us on the 1.92M-particle dam
+// break, 122.8 / 108.0 / 107.1 / 106.4 us on the 2.76M-particle collapse), 512 in
+// double (1562 / 1604 / 1671 / 1657 us at 1.36M particles).
+constexpr int kItemRound = 256;
+inline int32_t g2p_item_size(int64_t n, int num_sms, bool fp64)
+{
+    const int64_t q = (n / ((int64_t)num_sms * 4) + kItemRound - 1) / kItemRound * kItemRound, cap = fp64 ? 512 : 4096;
+    return (int32_t)(q < kItemRound ? kItemRound : (q > cap ? cap : q));
+}
 
 enum StatusBits { kStatusNaN = 1, kStatusChunkOverflow = 2, kStatusTimeout = 4 };
 

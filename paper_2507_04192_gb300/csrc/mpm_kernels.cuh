@@ -147,6 +147,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t phase)
 {
     uint32_t ok;
@@ -231,28 +235,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                      smem_u32(dst)),
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
-}
-
-// Stage the first ng components of the particle blocks covering slots
-// [a, a + count) (a a multiple of kPB) into a shared buffer, block after block
-// (ng kPB reals each: particle a + l's component c at buf[(l / kPB) ng kPB + c kPB
-// + l % kPB]).  Issued by warp 0: lane 0 sets the expected bytes, lane k copies
-// block k with one bulk copy.
-template <class R>
-__device__ __forceinline__ void stage_blocks(R *buf, const R *__restrict__ S, int ncomp, int ng, int64_t a, int count,
-                                             uint64_t *bar)
-{
-    const int nblk = (count + kPB - 1) / kPB;
-    const uint32_t bytes = (uint32_t)(ng * kPB * sizeof(R));
-    if (threadIdx.x < 32) {
-        if (threadIdx.x == 0) {
-            fence_proxy_async_smem();
-            mbar_expect_tx(bar, (uint32_t)nblk * bytes);
-        }
-        __syncwarp();
-        for (int k = threadIdx.x; k < nblk; k += 32)
-            bulk_g2s(buf + (int64_t)k * ng * kPB, S + ((a >> 5) + k) * (int64_t)ncomp * kPB, bytes, bar);
-    }
 }
 
 // ------------------------------------------------------------------ P2G
@@ -1650,140 +1632,143 @@ __device__ __forceinline__ bool g2p_particle(const Params<R> &P, Raw raw, R *__r
     return !bad && rfinite(chk);
 }
 
-// Shared-memory layout of the G2P block: the grid window, then two staging
-// buffers of NT / kPB particle blocks (the components G2P reads).
-// Particles per thread in one staged chunk of the G2P block (3D, 2D): chunks of 512
-// particles halve the block barriers per particle (3D dam break G2P 0.071 -> 0.067
-// ms, 2D batched 0.080 -> 0.074 ms; the 2.76M-particle collapse 0.118 -> 0.116).
-#ifndef MPM_G2P_PPT
-#define MPM_G2P_PPT 2
-#endif
-#ifndef MPM_G2P2_PPT
-#define MPM_G2P2_PPT 2
-#endif
-template <class R, int D> struct G2PSmem {
-    static constexpr int NT = 256;
-    static constexpr int CH = NT * (sizeof(R) == 4 ? (D == 3 ? MPM_G2P_PPT : MPM_G2P2_PPT) : 1);   // per chunk
-    static constexpr int NBLK = CH / kPB;
-    static constexpr int NCMAX = D + D * D + 8;
-    static constexpr size_t win_bytes = (size_t)Geo<D>::WN * sizeof(R4<R>);
-    static constexpr size_t buf_elems = (size_t)NBLK * NCMAX * kPB;
-    static constexpr size_t buf_bytes = 2 * buf_elems * sizeof(R);
-    static constexpr size_t total = win_bytes + buf_bytes + 128;
+// Shared-memory layout of the G2P block: two grid windows (the current work
+// item's and the next one's), then per warp two particle blocks of inputs.
+template <class R, int D, int MAT> struct G2PSmem {
+    static constexpr int NT = 256, NW = NT / 32;
+    static constexpr size_t win_elems = (size_t)(Geo<D>::WN + 7) / 8 * 8;       // whole 128-byte lines
+    static constexpr size_t win_bytes = win_elems * sizeof(R4<R>);
+    static constexpr size_t blk_elems = (size_t)Lay<D, MAT>::G2P_IN * kPB;
+    static constexpr size_t total = 2 * win_bytes + 2 * NW * blk_elems * sizeof(R) + 128;
 };
 
-// G2P of one tile t (compact list entry) by a block of NT threads: the tile's
-// velocity window by one TMA tensor copy, the particles in chunks of CH slots
-// aligned to the particle blocks, staged by bulk copies into two buffers of
-// buf_elems reals.  Returns false when a bounded wait ran out.
-template <class R, int D, bool GENERIC, int MAT, int NT, int CH>
-__device__ __forceinline__ bool g2p_tile(const Params<R> &P, const CUtensorMap *tmapV, R *__restrict__ S,
-                                         const R4<R> *__restrict__ V, const R4<R> *__restrict__ V2, int4 t,
-                                         R4<R> *Vw, R *bufs, size_t buf_elems, uint64_t *mbar, uint32_t &phases,
-                                         bool &bad)
-{
-    using Gm = Geo<D>;
-    using Ly = Lay<D, MAT>;
-    constexpr int nc = Ly::G2P_IN;
-    const int tid = threadIdx.x;
-    const int sim = (int)(t.x / P.tiles_per_sim);
-    int64_t tl = t.x - (int64_t)sim * P.tiles_per_sim;
-    int org[3] = {0, 0, 0};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        org[a] = (int)(tl % P.n_tiles[a]) * Gm::T;
-        tl /= P.n_tiles[a];
-    }
-    if (tid == 0 && !(P.debug & kDebugWithholdWindowCopy)) {
-        fence_proxy_async_smem();
-        mbar_expect_tx(&mbar[2], (uint32_t)(Gm::WN * sizeof(R4<R>)));
-        tma_load_window(Vw, tmapV, org, sim, D, &mbar[2]);
-    }
-    // particles in chunks of CH slots aligned to the particle blocks (so a warp's
-    // 32 particles are one block and each of its stores writes one line); slots
-    // of a neighbouring tile at either end are skipped
-    const int64_t a0 = (int64_t)t.y & ~(int64_t)(kPB - 1);
-    const int64_t pend = (int64_t)t.y + t.z;
-    const int nb = (int)((pend - a0 + CH - 1) / CH);
-    int cur = 0;
-    stage_blocks(bufs, S, Ly::NC, nc, a0, (int)(pend - a0 < CH ? pend - a0 : CH), &mbar[0]);
-    bool ok = mbar_wait_bounded(&mbar[2], (phases >> 2) & 1u);
-    phases ^= 4u;
-    const R4<R> *Vs = V + (int64_t)sim * P.nodes_per_sim;
-    const R4<R> *V2s = V2 != nullptr ? V2 + (int64_t)sim * P.nodes_per_sim : nullptr;
-    for (int j = 0; j < nb; ++j) {
-        if (j + 1 < nb) {
-            const int64_t an = a0 + (int64_t)(j + 1) * CH;
-            stage_blocks(bufs + (size_t)(cur ^ 1) * buf_elems, S, Ly::NC, nc, an,
-                         (int)(pend - an < CH ? pend - an : CH), &mbar[cur ^ 1]);
-        }
-        const bool okb = mbar_wait_bounded(&mbar[cur], (phases >> cur) & 1u);
-        phases ^= 1u << cur;
-        ok = ok && okb;
-#pragma unroll 1
-        for (int u = 0; u < CH / NT; ++u) {
-            const int l = u * NT + tid;                // slot within the chunk
-            const int64_t p = a0 + (int64_t)j * CH + l;
-            if (ok && p >= t.y && p < pend) {
-                const R *bb = bufs + (size_t)cur * buf_elems + (l >> 5) * (nc * kPB) + (l & (kPB - 1));
-                bad |= !g2p_particle<R, D, GENERIC, MAT>(P, [&](int jj) { return bb[jj * kPB]; }, S, p, Vw, org,
-                                                        Vs, V2s);
-            }
-        }
-        __syncthreads();
-        cur ^= 1;
-    }
-    return ok;
-}
-
-// G2P.  Blocks claim tiles dynamically, one thread per particle.  The tile's
-// grid window of velocities is staged by one TMA tiled load; the particles'
-// inputs are staged 256 at a time by TMA bulk copies, double-buffered.  All
-// waits are bounded; a timeout is reported in the status word.
+// G2P.  Persistent blocks take work items (runs of a tile's particles, the largest
+// first), one thread per particle; whole tiles as items left small problems on a
+// few blocks (a 50,560-particle sand cylinder: about 30 of them, 41.6 us per
+// launch, 8 us in runs of 256 particles).  A block's first item is its own index,
+// later ones come from the cursor.  The tile's grid window of velocities is staged
+// by one TMA tiled load, one item ahead; each warp stages its own 32-particle
+// blocks (w, w + 8, ... of the item) by one bulk copy each, one block ahead, and
+// never waits for the other warps: a window is refilled once all of them have
+// left its item (empty).  With block-wide chunks of 512 particles the block
+// barriers and the copies at the start of an item were exposed.  All waits
+// are bounded; a timeout is reported in the status word once the copies in flight
+// have landed.
 template <class R, int D, bool GENERIC, int MAT>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
     k_g2p(const Params<R> P, const __grid_constant__ CUtensorMap tmapV, R *__restrict__ S,
-          const R4<R> *__restrict__ V, const int4 *__restrict__ tiles, int32_t *__restrict__ counters,
+          const R4<R> *__restrict__ V, const int4 *__restrict__ items, int32_t *__restrict__ counters,
           int32_t *__restrict__ status, const R4<R> *__restrict__ V2)
 {
     using Gm = Geo<D>;
-    using L = G2PSmem<R, D>;
-    constexpr int NT = L::NT;
+    using L = G2PSmem<R, D, MAT>;
+    using Ly = Lay<D, MAT>;
+    constexpr int NW = L::NW;
+    static_assert(Ly::G2P_IN == g2p_ncomp<D>(MAT), "G2P inputs lead the particle state");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // 128-byte aligned start for the TMA window, by pointer arithmetic on the shared
     // array (an integer round trip would hide the address space from the compiler and
     // turn every shared access into a generic one)
     unsigned char *base = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    R4<R> *Vw = reinterpret_cast<R4<R> *>(base);
-    R *bufs = reinterpret_cast<R *>(base + L::win_bytes);
-    __shared__ __align__(8) uint64_t mbar[3];      // [0], [1]: particle buffers, [2]: grid window
-    __shared__ int s_slot;
-    const int tid = threadIdx.x;
-    using Ly = Lay<D, MAT>;
-    constexpr int nc = Ly::G2P_IN;                 // x, F, rho [, sigma, eps]: the first nc components
-    static_assert(nc == g2p_ncomp<D>(MAT), "G2P inputs lead the particle state");
+    R4<R> *const wins = reinterpret_cast<R4<R> *>(base);
+    __shared__ __align__(8) uint64_t full[2], empty[2], blk[NW][2];
+    __shared__ int4 s_item[2];                     // (simulation, tile coordinates, first particle, count)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    R *const bufs = reinterpret_cast<R *>(base + 2 * L::win_bytes) + (size_t)warp * 2 * L::blk_elems;
+    const bool withhold = (P.debug & kDebugWithholdWindowCopy) != 0;
+    const int n_items = counters[6];
+    int claim = n_items;                           // thread 0: the item after the published ones
+    auto take = [&]() { return n_items > (int)gridDim.x ? (int)gridDim.x + atomicAdd(&counters[3], 1) : n_items; };
+    auto publish = [&](int slot, int id) {         // thread 0: item id and its window to a slot (count 0: no more)
+        if (id >= n_items) {
+            s_item[slot] = make_int4(0, 0, 0, 0);
+            mbar_arrive(&full[slot]);
+            return;
+        }
+        const int4 t = items[id];
+        s_item[slot] = t;
+        if (withhold) return;
+        const int org[3] = {(t.y & 1023) * Gm::T, ((t.y >> 10) & 1023) * Gm::T, (t.y >> 20) * Gm::T};
+        fence_proxy_async_smem();
+        mbar_expect_tx(&full[slot], (uint32_t)(Gm::WN * sizeof(R4<R>)));
+        tma_load_window(wins + slot * L::win_elems, &tmapV, org, t.x, D, &full[slot]);
+    };
     if (tid == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
-        mbar_init(&mbar[2], 1);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], NW);
+            for (int v = 0; v < NW; ++v) mbar_init(&blk[v][i], 1);
+        }
         fence_mbar_init();
     }
-    uint32_t phases = 0u;                          // bit i: parity of the next wait on mbar[i]
+    __syncthreads();
+    if (tid == 0) {
+        publish(0, blockIdx.x);
+        publish(1, take());
+        claim = take();
+    }
     bool bad = false, timed_out = false;
-    const int n_tiles = counters[1];
-    for (;;) {
-        const int k = next_tile(&counters[3], n_tiles, &s_slot);
-        if (k < 0) break;
-        const int4 t = tiles[k];
-        const bool ok = g2p_tile<R, D, GENERIC, MAT, NT, L::CH>(P, &tmapV, S, V, V2, t, Vw, bufs, L::buf_elems, mbar,
-                                                             phases, bad);
-        timed_out |= !ok;
-        if (__syncthreads_or(timed_out)) {
-            if (tid == 0) atomicOr(status, (int32_t)kStatusTimeout);
+    uint32_t phases = 0u;                          // bit d: parity of the next wait on blk[warp][d]
+    for (int i = 0;; ++i) {
+        const int slot = i & 1;
+        const uint32_t ph = (uint32_t)(i >> 1) & 1u;
+        timed_out = !mbar_wait_bounded(&full[slot], ph);
+        if (__any_sync(0xffffffffu, timed_out)) {
+            timed_out = true;
+            if (!withhold) {                       // the windows in flight land before the block leaves
+                mbar_wait_bounded(&full[slot], ph);
+                mbar_wait_bounded(&full[slot ^ 1], (uint32_t)((i + 1) >> 1) & 1u);
+            }
+            break;
+        }
+        const int4 t = s_item[slot];
+        if (t.w == 0) break;
+        const int org[3] = {(t.y & 1023) * Gm::T, ((t.y >> 10) & 1023) * Gm::T, (t.y >> 20) * Gm::T};
+        const R4<R> *Vw = wins + slot * L::win_elems;
+        const int b1 = (t.z + t.w + kPB - 1) / kPB;            // particle blocks [t.z / kPB, b1)
+        auto stage = [&](int b, int d) {
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                mbar_expect_tx(&blk[warp][d], (uint32_t)(L::blk_elems * sizeof(R)));
+                bulk_g2s(bufs + d * L::blk_elems, S + (int64_t)b * Ly::NC * kPB, (uint32_t)(L::blk_elems * sizeof(R)),
+                         &blk[warp][d]);
+            }
+        };
+        int b = t.z / kPB + warp, d = 0;
+        if (b < b1) stage(b, 0);
+        if (b + NW < b1) stage(b + NW, 1);
+        for (; b < b1; b += NW, d ^= 1) {
+            if (!mbar_wait_bounded(&blk[warp][d], (phases >> d) & 1u)) timed_out = true;
+            phases ^= 1u << d;
+            const int p = b * kPB + lane;
+            if (!timed_out && p >= t.z && p < t.z + t.w) {
+                const R *bb = bufs + d * L::blk_elems + lane;
+                bad |= !g2p_particle<R, D, GENERIC, MAT>(P, [&](int jj) { return bb[jj * kPB]; }, S, p, Vw, org,
+                                                        V + (int64_t)t.x * P.nodes_per_sim,
+                                                        V2 != nullptr ? V2 + (int64_t)t.x * P.nodes_per_sim : nullptr);
+            }
+            __syncwarp();
+            if (b + 2 * NW < b1) stage(b + 2 * NW, d);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[slot]);
+        if (tid == 0) {                            // the next item but one, once every warp has left this window
+            if (!timed_out && mbar_wait_bounded(&empty[slot], ph)) {
+                publish(slot, claim);
+                if (claim < n_items) claim = take();
+            } else {
+                timed_out = true;
+            }
+        }
+        timed_out = __any_sync(0xffffffffu, timed_out);
+        if (timed_out) {                           // the next item's window lands before the block leaves
+            if (!withhold) mbar_wait_bounded(&full[slot ^ 1], (uint32_t)((i + 1) >> 1) & 1u);
             break;
         }
     }
-    if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) atomicOr(status, (int32_t)kStatusNaN);
+    if (timed_out && lane == 0) atomicOr(status, (int32_t)kStatusTimeout);
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, (int32_t)kStatusNaN);
     if (tid == 0) {
         counters[2] = 0;                           // P2G cursor for the next kernel (P2G follows)
         counters[4] = 0;                           // the grid update has walked the touched-tile list
@@ -2114,7 +2099,7 @@ template <class R, int D> struct Launch {
     template <bool GENERIC, int MAT> static void g2p_launch(const HostParams &h, DevState &ds)
     {
         auto P = make_params<R>(h, ds);
-        const size_t smem = G2PSmem<R, D>::total;
+        const size_t smem = G2PSmem<R, D, MAT>::total;
         static bool attr = false;
         if (!attr) {
             cudaFuncSetAttribute(k_g2p<R, D, GENERIC, MAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2124,17 +2109,17 @@ template <class R, int D> struct Launch {
         // per SM; 2D: three, its registers and shared memory allow it)
         static int per_sm = 0;
         if (per_sm == 0) {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<R, D, GENERIC, MAT>, G2PSmem<R, D>::NT,
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<R, D, GENERIC, MAT>, G2PSmem<R, D, MAT>::NT,
                                                               smem) != cudaSuccess ||
                 per_sm < 1)
                 per_sm = sizeof(R) == 4 ? MPM_G2P_MINB : 2;
         }
-        int64_t nb = ds.max_tiles;
+        int64_t nb = ds.max_items;
         const int64_t cap = (int64_t)ds.num_sms * per_sm;
         if (nb > cap) nb = cap;
         if (nb < 1) nb = 1;
-        k_g2p<R, D, GENERIC, MAT><<<(int)nb, G2PSmem<R, D>::NT, smem, ds.stream>>>(
-            P, ds.tmap_V, (R *)ds.S, (const R4<R> *)ds.V, ds.tiles + ds.max_tiles, ds.counters, ds.status,
+        k_g2p<R, D, GENERIC, MAT><<<(int)nb, G2PSmem<R, D, MAT>::NT, smem, ds.stream>>>(
+            P, ds.tmap_V, (R *)ds.S, (const R4<R> *)ds.V, ds.items, ds.counters, ds.status,
             (const R4<R> *)ds.V2);
     }
     static void g2p(const HostParams &h, DevState &ds)

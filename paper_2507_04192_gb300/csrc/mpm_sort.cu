@@ -235,22 +235,32 @@ __global__ void __launch_bounds__(1024) k_build_tiles(const int32_t *__restrict_
     if (threadIdx.x == 0) counters[1] = (int32_t)(carry < max_tiles ? carry : max_tiles);
 }
 
-// Copies the compact tile list, ordered by particle count with the largest
-// first, to tiles + max_tiles: the persistent G2P blocks claim tiles from that
-// copy in order and so finish together (longest-processing-time-first).  P2G
-// keeps the spatial order of the original list, whose neighbouring tiles share
-// the grid nodes of their windows.  Counting sort on buckets of 32 particles.
-__global__ void __launch_bounds__(1024) k_order_tiles(int4 *__restrict__ tiles, const int32_t *__restrict__ counters,
-                                                      int64_t max_tiles)
+// G2P's work items: every tile of the compact list cut into equal runs of at most
+// about q particles, cut at particle-block boundaries, the largest runs first, to
+// items[0 .. counters[6]): the persistent G2P blocks take them in order and so
+// finish together (longest-processing-time-first).  An item is (simulation, tile
+// coordinates in 10 bits each, first particle, count).  P2G keeps the spatial
+// order of the tile list, whose neighbouring tiles share grid nodes.  Counting
+// sort on buckets of 32 particles.
+__global__ void __launch_bounds__(1024) k_order_items(const int4 *__restrict__ tiles, int32_t *__restrict__ counters,
+                                                      int32_t q, int64_t tiles_per_sim, int ntx, int nty,
+                                                      int4 *__restrict__ items)
 {
     constexpr int NB = 128;
     __shared__ int32_t hist[NB];
     const int n = counters[1];
-    int4 *out = tiles + max_tiles;
     for (int b = threadIdx.x; b < NB; b += blockDim.x) hist[b] = 0;
     __syncthreads();
     auto bucket = [](int cnt) { return NB - 1 - min(cnt >> 5, NB - 1); };
-    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&hist[bucket(tiles[i].z)], 1);
+    // runs of tile t: boundaries at floor(t.y / kPB) kPB + k run, whole rounds of a block's eight warps
+    auto cut = [&](const int4 &t, auto &&emit) {
+        const int a0 = t.y & ~(kPB - 1), end = t.y + t.z, span = end - a0;
+        const int m = (span + q - 1) / q;
+        const int run = ((span + m - 1) / m + kItemRound - 1) / kItemRound * kItemRound;
+        for (int s = a0; s < end; s += run) emit(max(s, t.y), min(s + run, end));
+    };
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        cut(tiles[i], [&](int b, int e) { atomicAdd(&hist[bucket(e - b)], 1); });
     __syncthreads();
     if (threadIdx.x == 0) {
         int sum = 0;
@@ -259,11 +269,15 @@ __global__ void __launch_bounds__(1024) k_order_tiles(int4 *__restrict__ tiles, 
             hist[b] = sum;
             sum += h;
         }
+        counters[6] = sum;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int4 t = tiles[i];
-        out[atomicAdd(&hist[bucket(t.z)], 1)] = t;
+        const int sim = (int)(t.x / tiles_per_sim);
+        const int tl = (int)(t.x - sim * tiles_per_sim);
+        const int u = (tl % ntx) | ((tl / ntx % nty) << 10) | ((tl / ntx / nty) << 20);
+        cut(t, [&](int b, int e) { items[atomicAdd(&hist[bucket(e - b)], 1)] = make_int4(sim, u, b, e - b); });
     }
 }
 
@@ -413,7 +427,8 @@ void build_tiles(const HostParams &hp, DevState &ds)
                                                                  ds.tile_end);
     k_build_tiles<<<1, 1024, 0, ds.stream>>>(ds.tile_start, ds.tile_end, ntiles, ds.tiles, ds.max_tiles,
                                              ds.counters, ds.status);
-    k_order_tiles<<<1, 1024, 0, ds.stream>>>(ds.tiles, ds.counters, ds.max_tiles);
+    k_order_items<<<1, 1024, 0, ds.stream>>>(ds.tiles, ds.counters, ds.item_q, hp.tiles_per_sim, hp.n_tiles[0],
+                                             hp.n_tiles[1], ds.items);
     int64_t tb = ds.max_tiles < (int64_t)ds.num_sms * 8 ? ds.max_tiles : (int64_t)ds.num_sms * 8;
     if (tb < 1) tb = 1;
     if (hp.dim == 2)
