@@ -44,76 +44,147 @@ __global__ void k_transpose_bf16(const __nv_bfloat16 *__restrict__ in, __nv_bflo
     }
 }
 
-__device__ __forceinline__ float gelu_grad_f(float z)
+// Network input: bf16 rows and their transpose (cols x rows) in one pass; the step's
+// loss is cleared on the way.
+__global__ void __launch_bounds__(256) k_prepare_input(const float *__restrict__ x, __nv_bfloat16 *__restrict__ out,
+                                                       __nv_bfloat16 *__restrict__ outT, int rows, int cols,
+                                                       double *__restrict__ loss)
 {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+    __shared__ __nv_bfloat16 tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *loss = 0.0;
+    for (int j = ty; j < 32; j += 8) {
+        const int r = r0 + j, c = c0 + tx;
+        if (r < rows && c < cols) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(x[(int64_t)r * cols + c]);
+            tile[j][tx] = h;
+            out[(int64_t)r * cols + c] = h;
+        }
+    }
+    __syncthreads();
+    for (int j = ty; j < 32; j += 8) {
+        const int c = c0 + j, r = r0 + tx;
+        if (r < rows && c < cols) outT[(int64_t)c * rows + r] = tile[tx][j];
+    }
 }
 
-// Loss and output gradient: L = mean (y - t)^2; dz = dL/dy (hi - lo) s (1 - s)
-// (dz = dL/dy for the linear output).
-__global__ void k_mse_out(const float *__restrict__ y, const float *__restrict__ t, const float *__restrict__ z,
-                          float *__restrict__ dz, int64_t n, float lo, float hi, double *__restrict__ loss,
-                          int linear)
+// Gradient of the output layer's pre-activation, dz = g (hi - lo) s (1 - s) with s =
+// sigmoid(z) (dz = g for the linear output), in fp32, bf16 and transposed bf16.
+// With a loss pointer, src holds the targets, g = 2 (y - t) / n and the loss mean
+// (y - t)^2 is added up; else src holds g = dL/dy.
+__global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y, const float *__restrict__ src,
+                                                     const float *__restrict__ z, float *__restrict__ dz,
+                                                     __nv_bfloat16 *__restrict__ dzb, __nv_bfloat16 *__restrict__ dzbT,
+                                                     int rows, int cols, float lo, float hi, int linear,
+                                                     double *__restrict__ loss)
 {
+    __shared__ __nv_bfloat16 tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    const int64_t n = (int64_t)rows * cols;
     double acc = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float e = y[i] - t[i];
-        acc += (double)e * e;
-        if (linear) {
-            dz[i] = 2.0f * e / (float)n;
-        } else {
-            const float s = 1.0f / (1.0f + expf(-z[i]));
-            dz[i] = 2.0f * e / (float)n * (hi - lo) * s * (1.0f - s);
+    for (int j = ty; j < 32; j += 8) {
+        const int r = r0 + j, c = c0 + tx;
+        if (r >= rows || c >= cols) continue;
+        const int64_t i = (int64_t)r * cols + c;
+        float g = src[i];
+        if (loss != nullptr) {
+            const float e = y[i] - g;
+            acc += (double)e * e;
+            g = 2.0f * e / (float)n;
         }
+        if (!linear) {
+            const float s = 1.0f / (1.0f + expf(-z[i]));
+            g = g * (hi - lo) * s * (1.0f - s);
+        }
+        dz[i] = g;
+        const __nv_bfloat16 h = __float2bfloat16_rn(g);
+        dzb[i] = h;
+        tile[j][tx] = h;
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc / (double)n);
-}
-
-// dz_prev = da * GELU'(z_prev), or da * [z_prev > 0] for ReLU.
-__global__ void k_act_back(const float *__restrict__ da, const float *__restrict__ z, float *__restrict__ dz,
-                           int64_t n, int relu)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dz[i] = relu ? (z[i] > 0.0f ? da[i] : 0.0f) : da[i] * gelu_grad_f(z[i]);
-}
-
-// Output gradient from a given dL/dy: dz = dy (hi - lo) s (1 - s) for the scaled
-// sigmoid, dz = dy for the linear output.
-__global__ void k_out_back(const float *__restrict__ dy, const float *__restrict__ z, float *__restrict__ dz,
-                           int64_t n, float lo, float hi, int linear)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (linear) {
-            dz[i] = dy[i];
-        } else {
-            const float s = 1.0f / (1.0f + expf(-z[i]));
-            dz[i] = dy[i] * (hi - lo) * s * (1.0f - s);
-        }
+    if (loss != nullptr) {
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (tx == 0) atomicAdd(loss, acc / (double)n);
+    }
+    __syncthreads();
+    for (int j = ty; j < 32; j += 8) {
+        const int c = c0 + j, r = r0 + tx;
+        if (r < rows && c < cols) dzbT[(int64_t)c * rows + r] = tile[tx][j];
     }
 }
 
-// db[c] = sum_r dz[r][c].
-__global__ void k_col_sum(const float *__restrict__ dz, float *__restrict__ db, int rows, int cols)
+// The end of a training step over all layers, one launch (a training step was 38 small
+// launches: separate conversions, transposes, column sums on one block, activation
+// gradients, Adam and copies per layer; with those in the GEMM epilogues, k_output_grad
+// and here it is 9, and 310 -> 92 us at batch 256 on 640-256-256-32): the bias gradients db[c] =
+// sum_r dz[r][c] (blocks [0, n_bias), 32 columns each), and with update Adam on the
+// fp32 master parameters (bias-corrected moments) with the weights' bf16 copies and
+// transposes (32 x 32 tiles of the weights).
+constexpr int kMaxLayers = 8;
+struct StepEnd {
+    struct Layer {
+        float *W, *gW, *mW, *vW, *b, *gb, *mb, *vb;
+        const float *dZ;
+        __nv_bfloat16 *Wb, *WbT;
+        int rows, cols;                        // N x K of the weights
+        int bias0, tile0;                      // first block of the layer's biases, of its weight tiles
+    } layer[kMaxLayers];
+    int L, batch, n_bias;
+    float lr, c1, c2;
+    int update;
+    const double *loss;
+    double *loss_out;                          // when set, receives the step's loss
+};
+
+__device__ __forceinline__ float adam(float *p, float gi, float *m, float *v, const StepEnd &s)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += dz[(int64_t)r * cols + c];
-    db[c] = s;
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    const float mi = b1 * *m + (1.f - b1) * gi;
+    const float vi = b2 * *v + (1.f - b2) * gi * gi;
+    *m = mi;
+    *v = vi;
+    const float q = *p - s.lr * (mi / s.c1) / (sqrtf(vi / s.c2) + eps);
+    *p = q;
+    return q;
 }
 
-// Adam on fp32 master parameters (bias-corrected moments).
-__global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, int64_t n, float lr, float b1, float b2, float eps, float c1, float c2)
+__global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEnd s)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    __shared__ float tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, blk = blockIdx.x;
+    if (blk == 0 && threadIdx.x == 0 && s.loss_out != nullptr) *s.loss_out = *s.loss;
+    int l = 0;
+    if (blk < s.n_bias) {
+        while (l + 1 < s.L && blk >= s.layer[l + 1].bias0) ++l;
+        const StepEnd::Layer &y = s.layer[l];
+        const int c = (blk - y.bias0) * 32 + tx;
+        float sum = 0.f;
+        if (c < y.rows)
+            for (int r = ty; r < s.batch; r += 8) sum += y.dZ[(int64_t)r * y.rows + c];
+        tile[ty][tx] = sum;
+        __syncthreads();
+        if (ty == 0 && c < y.rows) {
+            for (int j = 1; j < 8; ++j) sum += tile[j][tx];
+            y.gb[c] = sum;
+            if (s.update) adam(y.b + c, sum, y.mb + c, y.vb + c, s);
+        }
+        return;
+    }
+    while (l + 1 < s.L && blk >= s.layer[l + 1].tile0) ++l;
+    const StepEnd::Layer &y = s.layer[l];
+    const int t = blk - y.tile0, tc = (y.cols + 31) / 32;
+    const int r0 = t / tc * 32, c0 = t % tc * 32;
+    for (int j = ty; j < 32; j += 8) {
+        const int r = r0 + j, c = c0 + tx;
+        if (r >= y.rows || c >= y.cols) continue;
+        const int64_t i = (int64_t)r * y.cols + c;
+        const float q = adam(y.W + i, y.gW[i], y.mW + i, y.vW + i, s);
+        y.Wb[i] = __float2bfloat16_rn(q);
+        tile[j][tx] = q;
+    }
+    __syncthreads();
+    for (int j = ty; j < 32; j += 8) {
+        const int c = c0 + j, r = r0 + tx;
+        if (r < y.rows && c < y.cols) y.WbT[(int64_t)c * y.rows + r] = __float2bfloat16_rn(tile[tx][j]);
     }
 }
 
@@ -133,7 +204,7 @@ struct mpm_mlp {
     std::vector<__nv_bfloat16 *> X, XT;                     // layer inputs (bf16) and transposes, l = 0..L-1
     std::vector<float *> Z, dZ;                             // pre-activations and their gradients (fp32)
     std::vector<__nv_bfloat16 *> dZb, dZbT;
-    float *Y = nullptr, *T = nullptr, *dA = nullptr, *X0f = nullptr;
+    float *Y = nullptr, *T = nullptr, *X0f = nullptr;
     double *loss = nullptr;
     int32_t *status = nullptr;
     int64_t step = 0;
@@ -160,13 +231,9 @@ void refresh_bf16(mpm_mlp *m, int l)
     k_transpose_bf16<<<tg, tb, 0, m->stream>>>(m->Wb[l], m->WbT[l], m->w[l + 1], m->w[l]);
 }
 
-void transpose(mpm_mlp *m, const __nv_bfloat16 *in, __nv_bfloat16 *out, int rows, int cols)
-{
-    dim3 tb(32, 8), tg((cols + 31) / 32, (rows + 31) / 32);
-    k_transpose_bf16<<<tg, tb, 0, m->stream>>>(in, out, rows, cols);
-}
-
-int forward(mpm_mlp *m, int B)
+// With train, the hidden layers' activations are also stored transposed (the weight
+// gradients contract over the batch).
+int forward(mpm_mlp *m, int B, bool train)
 {
     for (int l = 0; l < m->L; ++l) {
         const int K = m->w[l], N = m->w[l + 1];
@@ -176,6 +243,7 @@ int forward(mpm_mlp *m, int B)
         if (l + 1 < m->L) {
             epi.mode = m->hidden_act == MPM_ACT_RELU ? kEpiBiasRelu : kEpiBiasGelu;
             epi.xnext = m->X[l + 1];
+            if (train) epi.xnextT = m->XT[l + 1];
         } else {
             epi.mode = m->out_act == MPM_OUT_LINEAR ? kEpiBiasLinear : kEpiBiasSigmoid;
             epi.y = m->Y;
@@ -217,76 +285,80 @@ int sync_status(mpm_mlp *m)
     return MPM_OK;
 }
 
-int load_x(mpm_mlp *m, int B, const float *x, bool device)
+// Rows of floats at src on the device: src itself, or its copy in dev (host rows, and
+// device rows that kernels cannot read in place).
+const float *on_device(mpm_mlp *m, const float *src, float *dev, int64_t n, bool device)
 {
-    const int64_t n = (int64_t)B * m->w[0];
-    const float *src = x;
-    if (!device) {
-        if (cudaMemcpyAsync(m->X0f, x, sizeof(float) * n, cudaMemcpyHostToDevice, m->stream) != cudaSuccess)
-            return MPM_ECUDA;
-        src = m->X0f;
-    }
-    k_f32_to_bf16<<<blocks_for(n), 256, 0, m->stream>>>(src, m->X[0], n);
-    return MPM_OK;
+    if (device && (reinterpret_cast<uintptr_t>(src) & 3) == 0) return src;
+    if (cudaMemcpyAsync(dev, src, sizeof(float) * n, device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                        m->stream) != cudaSuccess)
+        return nullptr;
+    return dev;
 }
 
-// Back-propagation from dZ[L - 1] (already holding dL/dz of the output layer)
-// and, with update, one Adam step.
-int backward_update(mpm_mlp *m, int B, double lr, int update)
+// Back-propagation from the output layer's pre-activation gradient (dZ[L - 1] with its
+// bf16 forms) and, with update, one Adam step; loss_out: device copy of the loss.
+// Per layer one launch computes dW = dZ^T X and, for l > 0, dA = dZ W, whose epilogue
+// forms the layer below's dZ; then one launch ends the step.
+int backward_update(mpm_mlp *m, int B, double lr, int update, double *loss_out)
 {
     const int L = m->L;
     for (int l = L - 1; l >= 0; --l) {
-        const int Kin = m->w[l], N = m->w[l + 1];
-        const int64_t nz = (int64_t)B * N;
-        k_f32_to_bf16<<<blocks_for(nz), 256, 0, m->stream>>>(m->dZ[l], m->dZb[l], nz);
-        transpose(m, m->dZb[l], m->dZbT[l], B, N);          // N x B
-        transpose(m, m->X[l], m->XT[l], B, Kin);             // Kin x B
-        // dW = dZ^T X : (N x B) (Kin x B)^T
-        cudaError_t e = umma_gemm_tma(N, Kin, B, m->dZbT[l], B, m->XT[l], B, m->gW[l], Kin, UmmaEpi{}, m->status,
-                                      m->stream);
-        if (e != cudaSuccess) return MPM_ECUDA;
-        k_col_sum<<<(N + 255) / 256, 256, 0, m->stream>>>(m->dZ[l], m->gb[l], B, N);
+        const int K = m->w[l], N = m->w[l + 1];
+        UmmaGemm g[2];
+        g[0] = UmmaGemm{N, K, B, m->dZbT[l], B, m->XT[l], B, m->gW[l], K, UmmaEpi{}};
         if (l > 0) {
-            // dA = dZ W : (B x N) (Kin x N)^T
-            e = umma_gemm_tma(B, Kin, N, m->dZb[l], N, m->WbT[l], N, m->dA, Kin, UmmaEpi{}, m->status, m->stream);
-            if (e != cudaSuccess) return MPM_ECUDA;
-            k_act_back<<<blocks_for((int64_t)B * Kin), 256, 0, m->stream>>>(m->dA, m->Z[l - 1], m->dZ[l - 1],
-                                                                           (int64_t)B * Kin,
-                                                                           m->hidden_act == MPM_ACT_RELU);
+            UmmaEpi epi;
+            epi.mode = m->hidden_act == MPM_ACT_RELU ? kEpiReluBack : kEpiGeluBack;
+            epi.zprev = m->Z[l - 1];
+            epi.xnext = m->dZb[l - 1];
+            epi.xnextT = m->dZbT[l - 1];
+            g[1] = UmmaGemm{B, K, N, m->dZb[l], N, m->WbT[l], N, m->dZ[l - 1], K, epi};
         }
+        if (umma_gemm_tiles(g, l > 0 ? 2 : 1, m->status, m->stream) != cudaSuccess) return MPM_ECUDA;
     }
-    if (update) {
-        m->step++;
-        const float b1 = 0.9f, b2 = 0.999f;
-        const float c1 = 1.f - powf(b1, (float)m->step), c2 = 1.f - powf(b2, (float)m->step);
-        for (int l = 0; l < L; ++l) {
-            const int64_t nw = (int64_t)m->w[l + 1] * m->w[l], nb = m->w[l + 1];
-            k_adam<<<blocks_for(nw), 256, 0, m->stream>>>(m->W[l], m->gW[l], m->mW[l], m->vW[l], nw, (float)lr, b1, b2,
-                                                          1e-8f, c1, c2);
-            k_adam<<<blocks_for(nb), 256, 0, m->stream>>>(m->b[l], m->gb[l], m->mb[l], m->vb[l], nb, (float)lr, b1, b2,
-                                                          1e-8f, c1, c2);
-            refresh_bf16(m, l);
-        }
+    if (update) m->step++;
+    StepEnd s{};
+    s.L = L;
+    s.batch = B;
+    s.lr = (float)lr;
+    s.c1 = 1.f - powf(0.9f, (float)m->step);
+    s.c2 = 1.f - powf(0.999f, (float)m->step);
+    s.update = update != 0;
+    s.loss = m->loss;
+    s.loss_out = loss_out;
+    int blocks = 0;
+    for (int l = 0; l < L; ++l) {
+        s.layer[l] = StepEnd::Layer{m->W[l], m->gW[l], m->mW[l], m->vW[l], m->b[l], m->gb[l], m->mb[l], m->vb[l],
+                                    m->dZ[l], m->Wb[l], m->WbT[l], m->w[l + 1], m->w[l], blocks, 0};
+        blocks += (m->w[l + 1] + 31) / 32;
     }
+    s.n_bias = blocks;
+    for (int l = 0; l < L && update; ++l) {
+        s.layer[l].tile0 = blocks;
+        blocks += ((m->w[l + 1] + 31) / 32) * ((m->w[l] + 31) / 32);
+    }
+    k_step_end<<<blocks, 256, 0, m->stream>>>(s);
     return MPM_OK;
 }
 
-// Queue one training step on the mean squared error (no synchronisation).
-int train_queue(mpm_mlp *m, int B, const float *x, const float *target, double lr, int update, bool device)
+// Queue the forward pass and the back-propagation of batch rows x (no
+// synchronisation): of the mean squared error to the targets (with_loss), or of a
+// given dL/dy (src).
+int train_queue(mpm_mlp *m, int B, const float *x, const float *src, double lr, int update, bool device, bool with_loss,
+                double *loss_out)
 {
-    const int L = m->L;
-    int rc = load_x(m, B, x, device);
+    const int L = m->L, nin = m->w[0], nout = m->w[L];
+    const float *xd = on_device(m, x, m->X0f, (int64_t)B * nin, device);
+    const float *sd = on_device(m, src, m->T, (int64_t)B * nout, device);
+    if (!xd || !sd) return MPM_ECUDA;
+    k_prepare_input<<<dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream>>>(xd, m->X[0], m->XT[0], B, nin, m->loss);
+    int rc = forward(m, B, true);
     if (rc != MPM_OK) return rc;
-    const int64_t nout = (int64_t)B * m->w[L];
-    if (cudaMemcpyAsync(m->T, target, sizeof(float) * nout, device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        m->stream) != cudaSuccess)
-        return MPM_ECUDA;
-    rc = forward(m, B);
-    if (rc != MPM_OK) return rc;
-    cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream);
-    k_mse_out<<<blocks_for(nout), 256, 0, m->stream>>>(m->Y, m->T, m->Z[L - 1], m->dZ[L - 1], nout, m->lo, m->hi,
-                                                      m->loss, m->out_act == MPM_OUT_LINEAR);
-    rc = backward_update(m, B, lr, update);
+    k_output_grad<<<dim3((nout + 31) / 32, (B + 31) / 32), 256, 0, m->stream>>>(
+        m->Y, sd, m->Z[L - 1], m->dZ[L - 1], m->dZb[L - 1], m->dZbT[L - 1], B, nout, m->lo, m->hi,
+        m->out_act == MPM_OUT_LINEAR, with_loss ? m->loss : nullptr);
+    rc = backward_update(m, B, lr, update, loss_out);
     return rc != MPM_OK ? rc : check(m);
 }
 
@@ -334,8 +406,6 @@ int mpm_mlp_create(int n_layers, const int *widths, int max_batch, double out_lo
     resize(m->W); resize(m->b); resize(m->gW); resize(m->gb); resize(m->mW); resize(m->vW); resize(m->mb);
     resize(m->vb); resize(m->Wb); resize(m->WbT); resize(m->X); resize(m->XT); resize(m->Z); resize(m->dZ);
     resize(m->dZb); resize(m->dZbT);
-    int maxw = 0;
-    for (int l = 0; l <= L; ++l) maxw = std::max(maxw, widths[l]);
     for (int l = 0; l < L && rc == MPM_OK; ++l) {
         const size_t nw = (size_t)widths[l + 1] * widths[l], nb = widths[l + 1];
         rc = malloc_n(m, &m->W[l], nw);
@@ -357,7 +427,6 @@ int mpm_mlp_create(int n_layers, const int *widths, int max_batch, double out_lo
     }
     if (rc == MPM_OK) rc = malloc_n(m, &m->Y, (size_t)B * widths[L]);
     if (rc == MPM_OK) rc = malloc_n(m, &m->T, (size_t)B * widths[L]);
-    if (rc == MPM_OK) rc = malloc_n(m, &m->dA, (size_t)B * maxw);
     if (rc == MPM_OK) rc = malloc_n(m, &m->X0f, (size_t)B * widths[0]);
     if (rc == MPM_OK) rc = malloc_n(m, &m->loss, 1);
     if (rc == MPM_OK) rc = malloc_n(m, &m->status, 1);
@@ -380,7 +449,7 @@ void mpm_mlp_destroy(mpm_mlp *m)
     for (auto *vec : {&m->Wb, &m->WbT, &m->X, &m->XT, &m->dZb, &m->dZbT})
         for (__nv_bfloat16 *p : *vec)
             if (p) cudaFree(p);
-    for (void *p : {(void *)m->Y, (void *)m->T, (void *)m->dA, (void *)m->X0f, (void *)m->loss, (void *)m->status})
+    for (void *p : {(void *)m->Y, (void *)m->T, (void *)m->X0f, (void *)m->loss, (void *)m->status})
         if (p) cudaFree(p);
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     delete m;
@@ -434,8 +503,11 @@ int mpm_mlp_get_params(mpm_mlp *m, float *params, int which)
 int mpm_mlp_infer(mpm_mlp *m, int batch, const float *x, float *y, int device_ptrs)
 {
     if (!m || !x || !y || batch < 1 || batch > m->max_batch) return MPM_EINVAL;
-    int rc = load_x(m, batch, x, device_ptrs != 0);
-    if (rc == MPM_OK) rc = forward(m, batch);
+    const int64_t nx = (int64_t)batch * m->w[0];
+    const float *xd = on_device(m, x, m->X0f, nx, device_ptrs != 0);
+    if (!xd) return MPM_ECUDA;
+    k_f32_to_bf16<<<blocks_for(nx), 256, 0, m->stream>>>(xd, m->X[0], nx);
+    int rc = forward(m, batch, false);
     if (rc == MPM_OK) rc = check(m);
     if (rc != MPM_OK) return rc;
     const size_t n = (size_t)batch * m->w[m->L];
@@ -449,7 +521,7 @@ int mpm_mlp_train_step(mpm_mlp *m, int batch, const float *x, const float *targe
                        double *loss_out, int device_ptrs)
 {
     if (!m || !x || !target || batch < 8 || batch > m->max_batch || (batch % 8) || !(lr >= 0)) return MPM_EINVAL;
-    int rc = train_queue(m, batch, x, target, lr, update, device_ptrs != 0);
+    int rc = train_queue(m, batch, x, target, lr, update, device_ptrs != 0, true, nullptr);
     if (rc != MPM_OK) return rc;
     if (loss_out &&
         cudaMemcpyAsync(loss_out, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
@@ -462,9 +534,10 @@ int mpm_mlp_train_step_async(mpm_mlp *m, int batch, const float *x_dev, const fl
 {
     if (!m || !x_dev || !target_dev || batch < 8 || batch > m->max_batch || (batch % 8) || !(lr >= 0))
         return MPM_EINVAL;
-    int rc = train_queue(m, batch, x_dev, target_dev, lr, 1, true);
+    const bool direct = (reinterpret_cast<uintptr_t>(loss_dev) & 7) == 0;     // a store of the last kernel
+    int rc = train_queue(m, batch, x_dev, target_dev, lr, 1, true, true, direct ? loss_dev : nullptr);
     if (rc != MPM_OK) return rc;
-    if (loss_dev &&
+    if (!direct &&
         cudaMemcpyAsync(loss_dev, m->loss, sizeof(double), cudaMemcpyDeviceToDevice, m->stream) != cudaSuccess)
         return MPM_ECUDA;
     return MPM_OK;
@@ -473,18 +546,7 @@ int mpm_mlp_train_step_async(mpm_mlp *m, int batch, const float *x_dev, const fl
 int mpm_mlp_backward(mpm_mlp *m, int batch, const float *x, const float *dy, double lr, int update, int device_ptrs)
 {
     if (!m || !x || !dy || batch < 8 || batch > m->max_batch || (batch % 8) || !(lr >= 0)) return MPM_EINVAL;
-    const int L = m->L;
-    int rc = load_x(m, batch, x, device_ptrs != 0);
-    if (rc == MPM_OK) rc = forward(m, batch);
-    if (rc != MPM_OK) return rc;
-    const int64_t nout = (int64_t)batch * m->w[L];
-    if (cudaMemcpyAsync(m->T, dy, sizeof(float) * nout, device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        m->stream) != cudaSuccess)
-        return MPM_ECUDA;
-    k_out_back<<<blocks_for(nout), 256, 0, m->stream>>>(m->T, m->Z[L - 1], m->dZ[L - 1], nout, m->lo, m->hi,
-                                                       m->out_act == MPM_OUT_LINEAR);
-    rc = backward_update(m, batch, lr, update);
-    if (rc == MPM_OK) rc = check(m);
+    int rc = train_queue(m, batch, x, dy, lr, update, device_ptrs != 0, false, nullptr);
     return rc != MPM_OK ? rc : sync_status(m);
 }
 

@@ -8,6 +8,7 @@
 // records it in the status word, frees its TMEM and leaves.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -46,30 +47,42 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N)
 // refill it).  A final commit signals the epilogue, which reads TMEM and either
 // stores C or applies bias + GELU (bf16 copy for the next layer) or bias +
 // scaled sigmoid.  All waits are bounded.
-// Tile choice: 128 x 128 tiles through a ring of MPM_UMMA_STAGES stages; when N
-// >= 256 and the 128 x 256 tiles alone fill every SM (MPM_UMMA_WIDE), 128 x 256
-// tiles through MPM_UMMA_WIDE_STAGES stages (half the operand traffic per FLOP).
+// Tile choice (umma_gemm_tma): 128 x 256 tiles when they alone fill every SM (half the
+// operand traffic per FLOP), else 128 x 128, and narrower ones where 128 x 128 would
+// leave most SMs idle.
 #ifndef MPM_UMMA_STAGES
 #define MPM_UMMA_STAGES 4
-#endif
-#ifndef MPM_UMMA_WIDE
-#define MPM_UMMA_WIDE 1
 #endif
 #ifndef MPM_UMMA_WIDE_STAGES
 #define MPM_UMMA_WIDE_STAGES 4
 #endif
-// The 128 x 256 path as a persistent kernel with a double-buffered accumulator.
-#ifndef MPM_UMMA_PERSIST
-#define MPM_UMMA_PERSIST 1
-#endif
-enum UmmaEpilogue { kEpiStore = 0, kEpiBiasGelu = 1, kEpiBiasSigmoid = 2, kEpiBiasRelu = 3, kEpiBiasLinear = 4 };
+enum UmmaEpilogue {
+    kEpiStore = 0, kEpiBiasGelu = 1, kEpiBiasSigmoid = 2, kEpiBiasRelu = 3, kEpiBiasLinear = 4,
+    kEpiGeluBack = 5, kEpiReluBack = 6
+};
 
 struct UmmaEpi {
     int mode = kEpiStore;
     const float *bias = nullptr;      // N
-    __nv_bfloat16 *xnext = nullptr;   // kEpiBiasGelu / kEpiBiasRelu: bf16 GELU(z) / max(z, 0), ld = ldc
+    // kEpiBiasGelu / kEpiBiasRelu: bf16 GELU(z) / max(z, 0), ld = ldc; kEpiGeluBack /
+    // kEpiReluBack: the stored value in bf16.  xnextT: its transpose (N x M) when set.
+    __nv_bfloat16 *xnext = nullptr, *xnextT = nullptr;
     float *y = nullptr;               // kEpiBiasSigmoid: lo + (hi - lo) sigmoid(z); kEpiBiasLinear: z; ld = ldc
+    const float *zprev = nullptr;     // kEpiGeluBack / kEpiReluBack: C = acc GELU'(zprev) / acc [zprev > 0], ld = ldc
     float lo = 0.f, hi = 1.f;
+};
+
+// One GEMM of a launch: operands, output and its number of tiles (M fastest).
+struct alignas(64) UmmaJob {
+    CUtensorMap tmA, tmB;
+    float *C;
+    int M, N, K, ldc, tiles_m, tiles;
+    UmmaEpi epi;
+};
+// Up to two independent GEMMs in one launch: a small product fills a fraction of the
+// SMs, and the two of a network layer's backward pass need nothing from each other.
+struct UmmaJobs {
+    UmmaJob j[2];
 };
 
 // Shared-memory descriptor of a K-major tile written by TMA with 128-byte
@@ -102,20 +115,105 @@ __device__ __forceinline__ bool umma_wait_parity(uint64_t *bar, uint32_t parity)
 
 __device__ __forceinline__ float umma_gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 
-// The fused outputs of one accumulator value z (bias added) at offset o.
-__device__ __forceinline__ void umma_epi_outputs(const UmmaEpi &epi, int64_t o, float z)
+__device__ __forceinline__ float umma_gelu_grad(float z)
 {
-    if (epi.mode == kEpiBiasGelu) epi.xnext[o] = __float2bfloat16_rn(umma_gelu(z));
-    else if (epi.mode == kEpiBiasRelu) epi.xnext[o] = __float2bfloat16_rn(fmaxf(z, 0.0f));
-    else if (epi.mode == kEpiBiasSigmoid) epi.y[o] = epi.lo + (epi.hi - epi.lo) / (1.0f + expf(-z));
-    else if (epi.mode == kEpiBiasLinear) epi.y[o] = z;
+    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
+
+// Eight consecutive fp32 values (16-byte aligned when whole; else the first `left`).
+__device__ __forceinline__ void umma_row8(const float *src, bool whole, int left, float v[8])
+{
+    if (whole) {
+        const float4 a = reinterpret_cast<const float4 *>(src)[0], b = reinterpret_cast<const float4 *>(src)[1];
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = e < left ? src[e] : 0.f;
+}
+
+// Epilogue of one 8-column chunk of a row (this lane's): C and the fused outputs, in
+// 16-byte accesses where the chunk is whole and C's rows are 16-byte aligned.
+__device__ __forceinline__ void umma_store8(const uint32_t r[8], int row, int M, int col0, int N, float *Cout, int ldc,
+                                            const UmmaEpi &epi)
+{
+    const int64_t o0 = (int64_t)row * ldc + col0;
+    const bool whole = col0 + 8 <= N && (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(Cout) & 15) == 0;
+    float z[8], x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) z[e] = __uint_as_float(r[e]);
+    if (epi.mode == kEpiGeluBack || epi.mode == kEpiReluBack) {
+        float zv[8];
+        umma_row8(epi.zprev + o0, whole, N - col0, zv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float zp = zv[e];
+            z[e] = epi.mode == kEpiReluBack ? (zp > 0.0f ? z[e] : 0.0f) : z[e] * umma_gelu_grad(zp);
+            x[e] = z[e];
+        }
+    } else if (epi.mode != kEpiStore) {
+        float bv[8];
+        umma_row8(epi.bias + col0, whole, N - col0, bv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            z[e] += bv[e];
+            x[e] = epi.mode == kEpiBiasGelu      ? umma_gelu(z[e])
+                   : epi.mode == kEpiBiasRelu    ? fmaxf(z[e], 0.0f)
+                   : epi.mode == kEpiBiasSigmoid ? epi.lo + (epi.hi - epi.lo) / (1.0f + expf(-z[e]))
+                                                 : z[e];
+        }
+    }
+    if (whole) {
+        float4 *d = reinterpret_cast<float4 *>(Cout + o0);
+        d[0] = make_float4(z[0], z[1], z[2], z[3]);
+        d[1] = make_float4(z[4], z[5], z[6], z[7]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (col0 + e < N) Cout[o0 + e] = z[e];
+    }
+    if (epi.mode == kEpiStore) return;
+    if (epi.y != nullptr) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (col0 + e < N) epi.y[o0 + e] = x[e];
+    }
+    if (epi.xnext != nullptr) {
+        __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) h[e] = __float2bfloat16_rn(x[e]);
+        if (whole && (ldc & 7) == 0) {
+            *reinterpret_cast<uint4 *>(epi.xnext + o0) = *reinterpret_cast<const uint4 *>(h);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (col0 + e < N) epi.xnext[o0 + e] = h[e];
+        }
+        if (epi.xnextT != nullptr) {                 // 32 lanes: 32 consecutive rows of one column
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (col0 + e < N) epi.xnextT[(int64_t)(col0 + e) * M + row] = h[e];
+        }
+    }
+}
+
+// 16 accumulator columns of this warp's 32 TMEM lanes, without waiting for them.
+__device__ __forceinline__ void umma_ld16(uint32_t taddr, uint32_t r[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                 "%13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15])
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 template <int NT, int STAGES>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
-    k_umma_gemm_tma(int M, int N, int K, const __grid_constant__ CUtensorMap tmA,
-                    const __grid_constant__ CUtensorMap tmB, float *__restrict__ Cout, int ldc, UmmaEpi epi,
-                    int32_t *__restrict__ status)
+    k_umma_gemm_tma(const __grid_constant__ UmmaJobs jobs, int32_t *__restrict__ status)
 {
     static_assert(NT % 16 == 0 && NT >= 32 && NT <= 256, "tile width");
     constexpr int TMEM_COLS = NT <= 32 ? 32 : (NT <= 64 ? 64 : (NT <= 128 ? 128 : 256));
@@ -128,8 +226,12 @@ __global__ void __launch_bounds__(kUmmaThreads, 1)
     __shared__ uint32_t tmem_base;
     __shared__ int failed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kUmmaM, n0 = blockIdx.y * NT;
-    const int nk = (K + kUmmaKC - 1) / kUmmaKC;
+    const int second = (int)blockIdx.x >= jobs.j[0].tiles ? 1 : 0;
+    const UmmaJob &jb = jobs.j[second];
+    const int tile = (int)blockIdx.x - (second ? jobs.j[0].tiles : 0);
+    const int M = jb.M, N = jb.N;
+    const int m0 = tile % jb.tiles_m * kUmmaM, n0 = tile / jb.tiles_m * NT;
+    const int nk = (jb.K + kUmmaKC - 1) / kUmmaKC;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -166,12 +268,12 @@ __global__ void __launch_bounds__(kUmmaThreads, 1)
                          : "memory");
             asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
                          " [%0], [%1, {%2, %3}], [%4];" ::"r"(sa),
-                         "l"(reinterpret_cast<uint64_t>(&tmA)), "r"(kc * kUmmaKC), "r"(m0),
+                         "l"(reinterpret_cast<uint64_t>(&jb.tmA)), "r"(kc * kUmmaKC), "r"(m0),
                          "r"(umma_smem_u32(&full[s]))
                          : "memory");
             asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
                          " [%0], [%1, {%2, %3}], [%4];" ::"r"(sb),
-                         "l"(reinterpret_cast<uint64_t>(&tmB)), "r"(kc * kUmmaKC), "r"(n0),
+                         "l"(reinterpret_cast<uint64_t>(&jb.tmB)), "r"(kc * kUmmaKC), "r"(n0),
                          "r"(umma_smem_u32(&full[s]))
                          : "memory");
         }
@@ -211,26 +313,14 @@ __global__ void __launch_bounds__(kUmmaThreads, 1)
     const bool ok = __syncthreads_and(fin) && !failed;
     if (ok) {
         const int row = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < NT; c0 += 8) {
-            uint32_t r[8];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                           "=r"(r[7])
-                         : "r"(taddr)
-                         : "memory");
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        const UmmaEpi epi = jb.epi;
+        for (int c0 = 0; c0 < NT && n0 + c0 < N; c0 += 16) {
+            uint32_t r[16];
+            umma_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+            umma_wait_ld();
             if (row < M) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int col = n0 + c0 + e;
-                    if (col >= N) continue;
-                    float z = __uint_as_float(r[e]);
-                    const int64_t o = (int64_t)row * ldc + col;
-                    if (epi.mode != kEpiStore) z += epi.bias[col];
-                    Cout[o] = z;
-                    umma_epi_outputs(epi, o, z);
-                }
+                umma_store8(r, row, M, n0 + c0, N, jb.C, jb.ldc, epi);
+                if (n0 + c0 + 8 < N) umma_store8(r + 8, row, M, n0 + c0 + 8, N, jb.C, jb.ldc, epi);
             }
         }
     } else if (tid == 0) {
@@ -241,29 +331,6 @@ __global__ void __launch_bounds__(kUmmaThreads, 1)
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS)
                      : "memory");
-}
-
-// Epilogue of one 8-column chunk of a row: C (and the fused GELU / sigmoid outputs).
-__device__ __forceinline__ void umma_store8(const uint32_t r[8], int row, int col0, int N, float *Cout, int ldc,
-                                            const UmmaEpi &epi)
-{
-    const int64_t o0 = (int64_t)row * ldc + col0;
-    if (epi.mode == kEpiStore && col0 + 8 <= N && (ldc & 3) == 0) {     // two 16-byte stores
-        float4 *d = reinterpret_cast<float4 *>(Cout + o0);
-        d[0] = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
-        d[1] = make_float4(__uint_as_float(r[4]), __uint_as_float(r[5]), __uint_as_float(r[6]), __uint_as_float(r[7]));
-        return;
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const int col = col0 + e;
-        if (col >= N) continue;
-        float z = __uint_as_float(r[e]);
-        const int64_t o = o0 + e;
-        if (epi.mode != kEpiStore) z += epi.bias[col];
-        Cout[o] = z;
-        umma_epi_outputs(epi, o, z);
-    }
 }
 
 // Persistent, warp-specialised form for large problems: one CTA per SM walks the
@@ -431,7 +498,7 @@ __global__ void __launch_bounds__(kUmmaPersistThreads, 1)
                              : "r"(taddr)
                              : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (row < M && n0 + c0 < N) umma_store8(r, row, n0 + c0, N, Cout, ldc, epi);
+                if (row < M && n0 + c0 < N) umma_store8(r, row, M, n0 + c0, N, Cout, ldc, epi);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -475,24 +542,7 @@ inline bool umma_tensor_map(CUtensorMap *tm, const __nv_bfloat16 *ptr, int rows,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NT, int STAGES>
-inline cudaError_t umma_launch(int M, int N, int K, const CUtensorMap &tmA, const CUtensorMap &tmB, float *C, int ldc,
-                               const UmmaEpi &epi, int32_t *status, cudaStream_t stream)
-{
-    constexpr size_t smem = umma_tma_smem_bytes<NT, STAGES>();
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_umma_gemm_tma<NT, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
-    dim3 g((M + kUmmaM - 1) / kUmmaM, (N + NT - 1) / NT);
-    k_umma_gemm_tma<NT, STAGES><<<g, kUmmaThreads, smem, stream>>>(M, N, K, tmA, tmB, C, ldc, epi, status);
-    return cudaGetLastError();
-}
-
-// C = A B^T through the pipelined TMA kernel, with an optional fused epilogue.
-inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B,
-                                 int ldb, float *C, int ldc, const UmmaEpi &epi, int32_t *status, cudaStream_t stream)
+inline int umma_num_sms()
 {
     static int sms = 0;
     if (sms == 0) {
@@ -500,15 +550,80 @@ inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, in
         cudaGetDevice(&dev);
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
     }
-    const int NT = N <= 32 ? 32
-                   : (MPM_UMMA_WIDE && N >= 256 && (int64_t)((M + kUmmaM - 1) / kUmmaM) * ((N + 255) / 256) >= sms)
-                       ? 256
-                       : 128;
-    CUtensorMap tmA, tmB;
-    if (!umma_tensor_map(&tmA, A, M, K, lda, kUmmaM) || !umma_tensor_map(&tmB, B, N, K, ldb, NT))
-        return cudaErrorInvalidValue;
-    if (NT == 32) return umma_launch<32, 4>(M, N, K, tmA, tmB, C, ldc, epi, status, stream);
-    if (NT == 256 && MPM_UMMA_PERSIST) {
+    return sms;
+}
+
+// One GEMM C = A B^T of umma_gemm_tma / umma_gemm_pair.
+struct UmmaGemm {
+    int M, N, K;
+    const __nv_bfloat16 *A;
+    int lda;
+    const __nv_bfloat16 *B;
+    int ldb;
+    float *C;
+    int ldc;
+    UmmaEpi epi;
+};
+
+template <int NT, int STAGES>
+inline cudaError_t umma_launch(const UmmaGemm *g, int n, int32_t *status, cudaStream_t stream)
+{
+    constexpr size_t smem = umma_tma_smem_bytes<NT, STAGES>();
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(k_umma_gemm_tma<NT, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        attr = true;
+    }
+    UmmaJobs jobs;
+    int blocks = 0;
+    for (int i = 0; i < n; ++i) {
+        UmmaJob &j = jobs.j[i];
+        if (!umma_tensor_map(&j.tmA, g[i].A, g[i].M, g[i].K, g[i].lda, kUmmaM) ||
+            !umma_tensor_map(&j.tmB, g[i].B, g[i].N, g[i].K, g[i].ldb, NT))
+            return cudaErrorInvalidValue;
+        j.C = g[i].C;
+        j.M = g[i].M;
+        j.N = g[i].N;
+        j.K = g[i].K;
+        j.ldc = g[i].ldc;
+        j.epi = g[i].epi;
+        j.tiles_m = (j.M + kUmmaM - 1) / kUmmaM;
+        j.tiles = j.tiles_m * ((j.N + NT - 1) / NT);
+        blocks += j.tiles;
+    }
+    if (n == 1) jobs.j[1] = jobs.j[0];
+    k_umma_gemm_tma<NT, STAGES><<<blocks, kUmmaThreads, smem, stream>>>(jobs, status);
+    return cudaGetLastError();
+}
+
+// One or two GEMMs in tiles of the width that suits them: 32 or 64 columns where 128
+// would leave at least three quarters or half of the SMs without a tile (a tile's
+// epilogue, erff on every value, and its operand stream are then spread over more
+// SMs; the deeper ring covers the L2 latency of the short tiles: one row through
+// 640-256-256-32 with its copies 84 -> 60 us, its first GEMM alone was 17 us on two SMs).
+inline cudaError_t umma_gemm_tiles(const UmmaGemm *g, int n, int32_t *status, cudaStream_t stream)
+{
+    int64_t tiles = 0;
+    int widest = 0;
+    for (int i = 0; i < n; ++i) {
+        tiles += (int64_t)((g[i].M + kUmmaM - 1) / kUmmaM) * ((g[i].N + 127) / 128);
+        widest = g[i].N > widest ? g[i].N : widest;
+    }
+    const int sms = umma_num_sms();
+    if (widest <= 32 || 4 * tiles <= sms) return umma_launch<32, 8>(g, n, status, stream);
+    if (2 * tiles <= sms) return umma_launch<64, 8>(g, n, status, stream);
+    return umma_launch<128, MPM_UMMA_STAGES>(g, n, status, stream);
+}
+
+// C = A B^T through the pipelined TMA kernels, with an optional fused epilogue.
+inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B,
+                                 int ldb, float *C, int ldc, const UmmaEpi &epi, int32_t *status, cudaStream_t stream)
+{
+    const int sms = umma_num_sms();
+    if (N >= 256 && (int64_t)((M + kUmmaM - 1) / kUmmaM) * ((N + 255) / 256) >= sms) {
+        CUtensorMap tmA, tmB;
+        if (!umma_tensor_map(&tmA, A, M, K, lda, kUmmaM) || !umma_tensor_map(&tmB, B, N, K, ldb, 256))
+            return cudaErrorInvalidValue;
         constexpr size_t smem = umma_tma_smem_bytes<256, MPM_UMMA_WIDE_STAGES>();
         static bool attr = false;
         if (!attr) {
@@ -521,9 +636,8 @@ inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, in
             M, N, K, tmA, tmB, C, ldc, epi, status);
         return cudaGetLastError();
     }
-    if (NT == 256) return umma_launch<256, MPM_UMMA_WIDE_STAGES>(M, N, K, tmA, tmB, C, ldc, epi, status, stream);
-    return umma_launch<128, MPM_UMMA_STAGES>(M, N, K, tmA, tmB, C, ldc, epi, status, stream);
+    const UmmaGemm g{M, N, K, A, lda, B, ldb, C, ldc, epi};
+    return umma_gemm_tiles(&g, 1, status, stream);
 }
-
 
 }  // namespace mpm
