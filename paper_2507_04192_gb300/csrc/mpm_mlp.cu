@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
 // launches: separate conversions, transposes, column sums on one block, activation
 // gradients, Adam and copies per layer; with those in the GEMM epilogues, k_output_grad
 // and here it is 9, and 310 -> 92 us at batch 256 on 640-256-256-32): the bias gradients db[c] =
-// sum_r dz[r][c] (blocks [0, n_bias), 32 columns each), and with update Adam on the
+// sum_r dz[r][c], added in the order of the rows (blocks [0, n_bias), 32 columns each,
+// 256 rows at a time through shared memory), and with update Adam on the
 // fp32 master parameters (bias-corrected moments) with the weights' bf16 copies and
 // transposes (32 x 32 tiles of the weights).
 constexpr int kMaxLayers = 8;
@@ -149,6 +150,7 @@ __device__ __forceinline__ float adam(float *p, float gi, float *m, float *v, co
 
 __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEnd s)
 {
+    __shared__ float rows[256][32];
     __shared__ float tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, blk = blockIdx.x;
     if (blk == 0 && threadIdx.x == 0 && s.loss_out != nullptr) *s.loss_out = *s.loss;
@@ -158,12 +160,28 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
         const StepEnd::Layer &y = s.layer[l];
         const int c = (blk - y.bias0) * 32 + tx;
         float sum = 0.f;
-        if (c < y.rows)
-            for (int r = ty; r < s.batch; r += 8) sum += y.dZ[(int64_t)r * y.rows + c];
-        tile[ty][tx] = sum;
-        __syncthreads();
+        for (int r0 = 0; r0 < s.batch; r0 += 256) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int r = r0 + 8 * j + ty;
+                rows[8 * j + ty][tx] = r < s.batch && c < y.rows ? y.dZ[(int64_t)r * y.rows + c] : 0.f;
+            }
+            __syncthreads();
+            if (ty == 0) {                             // the loads ahead of the chain of sums
+                const int m = min(256, s.batch - r0);
+                int j = 0;
+                for (; j + 32 <= m; j += 32) {
+                    float v[32];
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) v[q] = rows[j + q][tx];
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) sum += v[q];
+                }
+                for (; j < m; ++j) sum += rows[j][tx];
+            }
+            __syncthreads();
+        }
         if (ty == 0 && c < y.rows) {
-            for (int j = 1; j < 8; ++j) sum += tile[j][tx];
             y.gb[c] = sum;
             if (s.update) adam(y.b + c, sum, y.mb + c, y.vb + c, s);
         }
