@@ -402,7 +402,7 @@ int load_particles(mpm_ctx *c, int64_t n, const double *x, const double *v, doub
     h.vol0 = particle_volume;
     h.mass = h.rho0 * particle_volume;
     const size_t rsz = c->grid.precision == MPM_FP64 ? 8 : 4;
-    const int nblk = (int)((n + kSortChunk - 1) / kSortChunk);
+    const int nblk = sort_blocks(n);
     {
         const int64_t all_tiles = (int64_t)c->grid.batch * h.tiles_per_sim;
         ds.max_tiles = all_tiles < n ? all_tiles : n;

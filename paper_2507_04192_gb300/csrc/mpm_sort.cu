@@ -22,17 +22,21 @@ __device__ __forceinline__ uint32_t lanemask_lt()
     return m;
 }
 
+// ITEMS keys per thread, loaded up front (their latencies overlap).
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_rs_hist(const uint32_t *__restrict__ keys, int64_t n,
                                                           int shift, uint32_t *__restrict__ hist, int nblk)
 {
     __shared__ uint32_t cnt[kRadixBins];
     for (int i = threadIdx.x; i < kRadixBins; i += blockDim.x) cnt[i] = 0u;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortChunk;
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = base + (int64_t)r * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & (kRadixBins - 1)], 1u);
-    }
+    const int64_t base = (int64_t)blockIdx.x * (ITEMS * kSortThreads) + threadIdx.x;
+    uint32_t key[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) key[r] = base + r * kSortThreads < n ? keys[base + r * kSortThreads] : 0u;
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+        if (base + r * kSortThreads < n) atomicAdd(&cnt[(key[r] >> shift) & (kRadixBins - 1)], 1u);
     __syncthreads();
     for (int d = threadIdx.x; d < kRadixBins; d += blockDim.x) hist[(int64_t)d * nblk + blockIdx.x] = cnt[d];
 }
@@ -121,6 +125,7 @@ __global__ void __launch_bounds__(1024) k_scan_down(uint32_t *__restrict__ data,
     block_scan_exclusive(data, b0, b1, partial[blockIdx.x]);
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const uint32_t *__restrict__ kin,
                                                              const int32_t *__restrict__ vin,
                                                              uint32_t *__restrict__ kout,
@@ -137,10 +142,19 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const uint32_t *__r
     }
     __syncthreads();
     const uint32_t lt = lanemask_lt();
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = (int64_t)blockIdx.x * kSortChunk + (int64_t)r * kSortThreads + tid;
-        const bool valid = i < n;
-        const uint32_t key = valid ? kin[i] : 0u;
+    const int64_t base = (int64_t)blockIdx.x * (ITEMS * kSortThreads) + tid;
+    uint32_t keys[ITEMS];
+    int32_t vals[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + r * kSortThreads;
+        keys[r] = i < n ? kin[i] : 0u;
+        vals[r] = i < n ? vin[i] : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const bool valid = base + r * kSortThreads < n;
+        const uint32_t key = keys[r];
         const uint32_t digit = (key >> shift) & (kRadixBins - 1);
         const uint32_t peers = __match_any_sync(0xffffffffu, valid ? digit : (uint32_t)kRadixBins);
         const uint32_t rank = __popc(peers & lt);
@@ -159,7 +173,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const uint32_t *__r
         if (valid) {
             const uint32_t pos = wcnt[warp][digit] + rank;
             kout[pos] = key;
-            vout[pos] = vin[i];
+            vout[pos] = vals[r];
         }
         __syncthreads();
         if (tid < kRadixBins)
@@ -178,7 +192,8 @@ __global__ void k_tile_bounds(const uint32_t *__restrict__ keys, int64_t n, int 
     }
 }
 
-// Block-wide exclusive scan (1024 threads) of one value per thread.
+// Block-wide exclusive scan (NW warps) of one value per thread.
+template <int NW>
 __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *warp_sum, int32_t &total)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -191,7 +206,7 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *warp
     if (lane == 31) warp_sum[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        const int32_t ws = warp_sum[lane];
+        const int32_t ws = lane < NW ? warp_sum[lane] : 0;
         int32_t wi = ws;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -223,7 +238,7 @@ __global__ void __launch_bounds__(1024) k_build_tiles(const int32_t *__restrict_
         const int32_t s = t < ntiles ? tstart[t] : -1;
         const int32_t cnt = s >= 0 ? tend[t] - s : 0;
         int32_t total;
-        const int32_t off = block_exclusive_scan(cnt > 0 ? 1 : 0, warp_sum, total);
+        const int32_t off = block_exclusive_scan<32>(cnt > 0 ? 1 : 0, warp_sum, total);
         if (cnt > 0) {
             const int64_t idx = carry + off;
             if (idx < max_tiles) tiles[idx] = make_int4((int32_t)t, s, cnt, (int32_t)idx);
@@ -290,91 +305,60 @@ __global__ void __launch_bounds__(1024) k_order_items(const int4 *__restrict__ t
 // and rank r lands at
 //     off[g NG] + sum_{r' < r} T_g(r') + #{l' < l : cnt[g NG + l'] > r}
 // where off is the exclusive prefix of the cell counts and T_g(r') the number
-// of cells of group g holding more than r' particles.  One block of NG threads per
-// tile; writes the gather permutation, the position map (slot of each
-// (cell, rank) particle) and the per-tile cell offsets.
+// of cells of group g holding more than r' particles.  One block per tile, a thread
+// per cell; the groups walk their ranks side by side, each with a barrier of its own
+// (one group after another: 18.0 us for 50,560 particles, 6.7 us so); writes the gather permutation, the position map
+// (slot of each (cell, rank) particle) and the per-tile cell offsets.
 template <int TN, int NG>
-__global__ void __launch_bounds__(NG) k_tile_reorder(const int4 *__restrict__ tiles,
+__global__ void __launch_bounds__(TN) k_tile_reorder(const int4 *__restrict__ tiles,
                                                      const int32_t *__restrict__ counters,
                                                      const uint32_t *__restrict__ keys,
                                                      const int32_t *__restrict__ vals, int32_t *__restrict__ perm,
                                                      int32_t *__restrict__ posmap, int32_t *__restrict__ cell_off)
 {
-    constexpr int NW = NG / 32;
-    constexpr int PER = TN / NG;
+    constexpr int NW = TN / 32, GW = NG / 32;        // warps of the block, of a group
     __shared__ int32_t cnt[TN];
     __shared__ int32_t cst[TN + 1];
-    __shared__ int32_t wsum[NW + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int32_t wsum[33];
+    __shared__ int32_t plane[2][NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = tid / NG;
     const int n_tiles = counters[1];
     for (int k = blockIdx.x; k < n_tiles; k += gridDim.x) {
         const int4 t = tiles[k];
         const int32_t start = t.y, count = t.z;
-        for (int c = tid; c < TN; c += NG) cnt[c] = 0;
+        cnt[tid] = 0;
         __syncthreads();
-        for (int i = tid; i < count; i += NG) atomicAdd(&cnt[keys[start + i] & (TN - 1)], 1);
+        for (int i = tid; i < count; i += TN) atomicAdd(&cnt[keys[start + i] & (TN - 1)], 1);
         __syncthreads();
-        // exclusive prefix of the counts over the TN cells (PER consecutive cells per thread)
-        {
-            int32_t v[PER], local = 0;
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                v[j] = cnt[tid * PER + j];
-                local += v[j];
-            }
-            int32_t incl = local;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t x = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += x;
-            }
-            if (lane == 31) wsum[warp] = incl;
-            __syncthreads();
-            if (tid == 0) {
-                int32_t run = 0;
-                for (int w = 0; w < NW; ++w) {
-                    const int32_t x = wsum[w];
-                    wsum[w] = run;
-                    run += x;
-                }
-                wsum[NW] = run;
-            }
-            __syncthreads();
-            int32_t run = wsum[warp] + incl - local;
-#pragma unroll
-            for (int j = 0; j < PER; ++j) {
-                cst[tid * PER + j] = run;
-                run += v[j];
-            }
-            if (tid == 0) cst[TN] = wsum[NW];
-            __syncthreads();
-        }
+        const int32_t my = cnt[tid];
+        int32_t total;
+        const int32_t mine = block_exclusive_scan<NW>(my, wsum, total);   // exclusive prefix of the counts
+        cst[tid] = mine;
+        if (tid == 0) cst[TN] = total;
+        __syncthreads();
         const uint32_t lt = (1u << lane) - 1u;
-        for (int g = 0; g < TN / NG; ++g) {
-            const int c = g * NG + tid;
-            const int32_t my = cnt[c];
-            const int32_t gbase = cst[g * NG];
-            int32_t R = 0;
-            for (int r = 0;; ++r) {
-                const bool pred = my > r;
-                const int32_t T = __syncthreads_count(pred);
-                if (T == 0) break;
-                const uint32_t ball = __ballot_sync(0xffffffffu, pred);
-                if (lane == 0) wsum[warp] = __popc(ball);
-                __syncthreads();
-                int32_t before = 0;
-                for (int w = 0; w < warp; ++w) before += wsum[w];
-                if (pred) {
-                    const int32_t pos = gbase + R + before + __popc(ball & lt);
-                    perm[start + pos] = vals[start + cst[c] + r];
-                    posmap[start + cst[c] + r] = pos;
-                }
-                R += T;
-                __syncthreads();
+        int32_t at = cst[g * NG];                        // start of the rank plane
+        for (int r = 0;; ++r) {
+            const uint32_t ball = __ballot_sync(0xffffffffu, my > r);
+            if (lane == 0) plane[r & 1][warp] = __popc(ball);
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(NG) : "memory");
+            int32_t before = 0, T = 0;
+#pragma unroll
+            for (int w = 0; w < GW; ++w) {
+                const int32_t c = plane[r & 1][g * GW + w];
+                before += g * GW + w < warp ? c : 0;
+                T += c;
             }
+            if (T == 0) break;
+            if (my > r) {
+                const int32_t pos = at + before + __popc(ball & lt);
+                perm[start + pos] = vals[start + mine + r];
+                posmap[start + mine + r] = pos;
+            }
+            at += T;
         }
         int32_t *co = cell_off + (int64_t)k * (TN + 1);
-        for (int c = tid; c <= TN; c += NG) co[c] = cst[c];
+        for (int c = tid; c <= TN; c += TN) co[c] = cst[c];
         __syncthreads();
     }
 }
@@ -388,7 +372,7 @@ void scan_exclusive(uint32_t *data, int64_t len, uint32_t *partial, cudaStream_t
     seg = (seg + 4095) / 4096 * 4096;
     if (seg < 4096) seg = 4096;
     const int nseg = (int)((len + seg - 1) / seg);
-    if (nseg <= 1) {
+    if (len <= kRadixBins * 64) {                      // four rounds of one block cost less than three launches
         k_scan_top<<<1, 1024, 0, stream>>>(data, (int)len);
         return;
     }
@@ -397,18 +381,25 @@ void scan_exclusive(uint32_t *data, int64_t len, uint32_t *partial, cudaStream_t
     k_scan_down<<<nseg, 1024, 0, stream>>>(data, len, seg, partial);
 }
 
-void radix_sort_pairs(const HostParams &hp, DevState &ds)
+template <int ITEMS> static int radix_passes(const HostParams &hp, DevState &ds)
 {
     const int64_t n = hp.n;
-    const int nblk = (int)((n + kSortChunk - 1) / kSortChunk);
+    const int nblk = sort_blocks(n);
     int cur = 0;
     for (int shift = 0; shift < ds.key_bits; shift += kRadixBits) {
-        k_rs_hist<<<nblk, kSortThreads, 0, ds.stream>>>(ds.keys[cur], n, shift, ds.hist, nblk);
+        k_rs_hist<ITEMS><<<nblk, kSortThreads, 0, ds.stream>>>(ds.keys[cur], n, shift, ds.hist, nblk);
         scan_exclusive(ds.hist, (int64_t)kRadixBins * nblk, ds.hist + (int64_t)kRadixBins * nblk, ds.stream);
-        k_rs_scatter<<<nblk, kSortThreads, 0, ds.stream>>>(ds.keys[cur], ds.vals[cur], ds.keys[cur ^ 1],
-                                                           ds.vals[cur ^ 1], n, shift, ds.hist, nblk);
+        k_rs_scatter<ITEMS><<<nblk, kSortThreads, 0, ds.stream>>>(ds.keys[cur], ds.vals[cur], ds.keys[cur ^ 1],
+                                                                  ds.vals[cur ^ 1], n, shift, ds.hist, nblk);
         cur ^= 1;
     }
+    return cur;
+}
+
+void radix_sort_pairs(const HostParams &hp, DevState &ds)
+{
+    const int cur = sort_items(hp.n) == kSortItemsSmall ? radix_passes<kSortItemsSmall>(hp, ds)
+                                                        : radix_passes<kSortItems>(hp, ds);
     if (cur == 1) {
         uint32_t *tk = ds.keys[0]; ds.keys[0] = ds.keys[1]; ds.keys[1] = tk;
         int32_t *tv = ds.vals[0]; ds.vals[0] = ds.vals[1]; ds.vals[1] = tv;
@@ -432,10 +423,10 @@ void build_tiles(const HostParams &hp, DevState &ds)
     int64_t tb = ds.max_tiles < (int64_t)ds.num_sms * 8 ? ds.max_tiles : (int64_t)ds.num_sms * 8;
     if (tb < 1) tb = 1;
     if (hp.dim == 2)
-        k_tile_reorder<Geo<2>::TN, Geo<2>::NG><<<(int)tb, Geo<2>::NG, 0, ds.stream>>>(
+        k_tile_reorder<Geo<2>::TN, Geo<2>::NG><<<(int)tb, Geo<2>::TN, 0, ds.stream>>>(
             ds.tiles, ds.counters, ds.keys[0], ds.vals[0], ds.perm, ds.posmap, ds.cell_off);
     else
-        k_tile_reorder<Geo<3>::TN, Geo<3>::NG><<<(int)tb, Geo<3>::NG, 0, ds.stream>>>(
+        k_tile_reorder<Geo<3>::TN, Geo<3>::NG><<<(int)tb, Geo<3>::TN, 0, ds.stream>>>(
             ds.tiles, ds.counters, ds.keys[0], ds.vals[0], ds.perm, ds.posmap, ds.cell_off);
     cudaMemsetAsync(ds.counters + 2, 0, 2 * sizeof(int32_t), ds.stream);   // tile cursors
 }
