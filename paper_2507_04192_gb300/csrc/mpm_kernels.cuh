@@ -1843,49 +1843,50 @@ __global__ void k_permute(int ncomp, int64_t n, int64_t npad, const R *__restric
     }
 }
 
-// Field readback in load order (doubles).
-template <class R, int D>
-__global__ void k_get_field(const Params<R> P, const R *__restrict__ S, const int32_t *__restrict__ id,
-                            int field, double *__restrict__ out)
+// Field readback in load order (doubles), WD values per particle.  A block converts 256
+// slots into shared memory and writes them value by value, consecutive lanes the
+// consecutive values of a particle: one thread per particle stored each of its values
+// WD doubles from its neighbour's, a sector per store (seven fields of 2.76M particles
+// 735 us, 293 us so).
+template <class R, int D, int WD>
+__global__ void __launch_bounds__(256) k_get_field(const Params<R> P, const R *__restrict__ S,
+                                                   const int32_t *__restrict__ id, int field, double *__restrict__ out)
 {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P.n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = id[p];
-        const R *Sp = S + sblock(p, P.ncomp);
-        switch (field) {
-        case 0:
-            for (int a = 0; a < D; ++a) out[o * D + a] = (double)Sp[(P.off_x + a) * kPB];
-            break;
-        case 1:
-            for (int a = 0; a < D; ++a) out[o * D + a] = (double)Sp[(P.off_v + a) * kPB];
-            break;
-        case 2:
-            for (int q = 0; q < D * D; ++q) out[o * D * D + q] = (double)Sp[(P.off_C + q) * kPB];
-            break;
-        case 3:
-            for (int q = 0; q < D * D; ++q) out[o * D * D + q] = (double)Sp[(P.off_F + q) * kPB];
-            break;
-        case 4:
-            out[o] = (double)Sp[P.off_rho * kPB];
-            break;
-        case 5: {
-            double s9[9];
-            if (P.material == 0) {
-                const double pr = (double)tait(P, Sp[P.off_rho * kPB]);
-                for (int q = 0; q < 9; ++q) s9[q] = (q % 4 == 0) ? -pr : 0.0;
+    constexpr int NT = 256;
+    __shared__ double val[NT * WD];
+    __shared__ int32_t ids[NT];
+    const int tid = threadIdx.x;
+    for (int64_t p0 = (int64_t)blockIdx.x * NT; p0 < P.n; p0 += (int64_t)gridDim.x * NT) {
+        const int64_t p = p0 + tid;
+        const int count = (int)(P.n - p0 < NT ? P.n - p0 : NT);
+        if (p < P.n) {
+            ids[tid] = id[p];
+            const R *Sp = S + sblock(p, P.ncomp);
+            double *v = val + tid * WD;
+            if (WD == 9 && field == 5) {               // the stress as 3 x 3
+                if (P.material == 0) {
+                    const double pr = (double)tait(P, Sp[P.off_rho * kPB]);
+                    for (int q = 0; q < WD; ++q) v[q] = (q % 4 == 0) ? -pr : 0.0;
+                } else {
+                    const int map[9] = {0, 3, 4, 3, 1, 5, 4, 5, 2};
+#pragma unroll
+                    for (int q = 0; q < WD; ++q) v[q] = (double)Sp[(P.off_sig + map[q % 9]) * kPB];
+                }
+            } else if (field == 6 && P.material == 0) {
+                v[0] = 0.0;
             } else {
-                const int map[9] = {0, 3, 4, 3, 1, 5, 4, 5, 2};
-                for (int q = 0; q < 9; ++q) s9[q] = (double)Sp[(P.off_sig + map[q]) * kPB];
+                const int off = field == 0 ? P.off_x : field == 1 ? P.off_v : field == 2 ? P.off_C
+                              : field == 3 ? P.off_F : field == 4 ? P.off_rho : P.off_eps;
+#pragma unroll
+                for (int q = 0; q < WD; ++q) v[q] = (double)Sp[(off + q) * kPB];
             }
-            for (int q = 0; q < 9; ++q) out[o * 9 + q] = s9[q];
-            break;
         }
-        case 6:
-            out[o] = P.material == 1 ? (double)Sp[P.off_eps * kPB] : 0.0;
-            break;
-        default:
-            break;
+        __syncthreads();
+        for (int e = tid; e < count * WD; e += NT) {
+            const int j = e / WD;
+            out[(int64_t)ids[j] * WD + (e - j * WD)] = val[e];
         }
+        __syncthreads();
     }
 }
 
@@ -2135,8 +2136,14 @@ template <class R, int D> struct Launch {
     static void get_field(const HostParams &h, DevState &ds, int field, double *out)
     {
         auto P = make_params<R>(h, ds);
-        k_get_field<R, D><<<grid_blocks(h.n, 256, ds.num_sms), 256, 0, ds.stream>>>(P, (const R *)ds.S, ds.id,
-                                                                                    field, out);
+        const int nb = grid_blocks(h.n, 256, ds.num_sms);
+        auto launch = [&](auto width) {
+            k_get_field<R, D, decltype(width)::value><<<nb, 256, 0, ds.stream>>>(P, (const R *)ds.S, ds.id, field, out);
+        };
+        if (field <= 1) launch(std::integral_constant<int, D>{});
+        else if (field <= 3) launch(std::integral_constant<int, D * D>{});
+        else if (field == 5) launch(std::integral_constant<int, 9>{});
+        else launch(std::integral_constant<int, 1>{});
     }
     static void set_field(const HostParams &h, DevState &ds, int field, const double *in)
     {
