@@ -1464,8 +1464,11 @@ template <class R, int D> struct AdjLaunch {
                     static_assert(smem <= 48 * 1024, "k_p2g_direct shared memory above the default limit");
                     P2GIO<R> io{(const R *)st, (const R *)a.coef, h.n, a.tiles, a.n_tiles, a.cursor, a.posmap,
                                 a.cell_off, (R4<R> *)a.GVB, nullptr};
-                    k_p2g_direct<R, 3, NT, 2><<<ds.num_sms * MPM_P2G_MINB, NT, smem, ds.stream>>>(P, io, nullptr,
-                                                                                               nullptr);
+                    const int nb = ds.num_sms * MPM_P2G_MINB;
+                    if (p2g_share<3>(h.n, ds.num_sms))
+                        k_p2g_direct<R, 3, NT, 2, kShareLanes<3>><<<nb, NT, smem, ds.stream>>>(P, io, nullptr, nullptr);
+                    else
+                        k_p2g_direct<R, 3, NT, 2, 1><<<nb, NT, smem, ds.stream>>>(P, io, nullptr, nullptr);
                 }
             } else {
                 k_adj_g2p_bwd3<R, false><<<pblocks(h, ds), 256, 0, ds.stream>>>(

@@ -833,89 +833,98 @@ template <int D, int MAT> __host__ __device__ constexpr int direct_stage_comps()
 {
     return MAT == 2 ? 24 : kP2GStageComps<D>;
 }
-// Per warp of k_p2g_direct: its work item's 129 cell offsets (padded to 132),
-// staged in shared memory at the start of the item.
-constexpr int kDirectOffPad = 132;
-// Cells per work item and cp.async stages per thread of the cell-ordered P2G.
-// Items of 32 cells give each lane one cell (its cursor walks that cell's
-// particles only) and more items to balance the SMs: on the 2.76M-particle
-// collapse P2G 0.123 ms with 128-cell items (four cells per lane), 0.118 with 64,
-// 0.105 with 32; on the batched 2D dam breaks 0.167 -> 0.152 ms.  In 2D (16
-// particles per cell in the dense fluids) the pipeline is one stage deeper.
-#ifndef MPM_P2G2_CELLS
-#define MPM_P2G2_CELLS 32
-#endif
+// Per warp of k_p2g_direct: two work items (the current and the next one), each its
+// cell offsets (at most 33) and, from kDirectTile on, its tile key, the tile's first
+// particle and its number.
+constexpr int kDirectItemInts = 40, kDirectTile = 36;
+// A work item of the cell-ordered P2G has 32 / G cells, G lanes for each (p2g_share): one
+// cell per lane in large problems (on the 2.76M-particle collapse P2G 0.123 ms with
+// 128-cell items, four cells per lane, 0.118 with 64, 0.105 with 32; on the batched 2D
+// dam breaks 0.167 -> 0.152 ms).  cp.async stages per thread: in 2D (16 particles per
+// cell in the dense fluids) one more.
 #ifndef MPM_P2G2_STAGES
 #define MPM_P2G2_STAGES 3
-#endif
-#ifndef MPM_P2G3_CELLS
-#define MPM_P2G3_CELLS 32
 #endif
 #ifndef MPM_P2G3_STAGES
 #define MPM_P2G3_STAGES 2
 #endif
-template <int D> __host__ __device__ constexpr int direct_cells() { return D == 3 ? MPM_P2G3_CELLS : MPM_P2G2_CELLS; }
 template <int D> __host__ __device__ constexpr int direct_stages() { return D == 3 ? MPM_P2G3_STAGES : MPM_P2G2_STAGES; }
 template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t p2g_direct_smem()
 {
     return (size_t)direct_stages<D>() * direct_stage_comps<D, MAT>() * NT * sizeof(R) +
-           (size_t)(NT / 32) * kDirectOffPad * sizeof(int32_t);
+           (size_t)(NT / 32) * 2 * kDirectItemInts * sizeof(int32_t);
 }
 
 // P2G without a shared-memory window (register accumulation, single precision).
-// Warps claim work items of 128 cells (two layer groups of a 3D tile, half of a
-// 2D tile) from a global cursor and never synchronise with each other: lane l
-// walks cells base + l, + 32, + 64, + 96 through a two-stage cp.async pipeline,
-// sums the particles still in their cell in registers and adds the 3^D node sums
-// of a cell straight to the grid with vector atomics (27 per cell in 3D instead
-// of 108 shared-memory atomics plus the window pass); particles that left their
-// cell are scattered on their own.  The warp marks the node tiles its cells reach.
+// A work item is 32 / G cells of a tile.  Warps take items from a global cursor and
+// never synchronise with each other: each lane walks its cell's particles (with G > 1
+// every G-th of them) through a cp.async pipeline and sums those still in their cell in
+// registers; the G lanes of a cell share out its 3^D nodes by halving exchanges
+// (share_nodes), and the node sums go straight to the grid with vector atomics (27 per
+// cell in 3D instead of 108 shared-memory atomics plus the window pass); particles that
+// left their cell are scattered on their own.  The warp marks the node tiles its cells
+// reach.
 #ifndef MPM_P2G_DIRECT
 #define MPM_P2G_DIRECT 1
 #endif
-// One work item of the cell-ordered P2G: the CELLS cells [cbase, cbase + CELLS)
-// of compact tile k (key order), one warp, lane l walking cells cbase + l + 32 r.
-// stg: this block's cp.async staging slots (ST stages x NCM x NT reals); s_off:
-// this warp's 132 shared ints for the item's cell offsets.  MAT 2 (the adjoint's
+// One round of the exchange between the lanes of a cell: of its node sums acc[0 .. N)
+// this lane keeps the lower half (or the upper one, where its bit of the lane index is
+// set), adds its partner's to it and moves it to acc[0 .. (N + 1) / 2).  first and
+// count (the sums' first node and their number) follow.
+template <int N, int NN, class R, int NV>
+__device__ __forceinline__ void share_nodes(R (&acc)[NN][NV], int bit, int &first, int &count)
+{
+    constexpr int H = (N + 1) / 2;
+    static_assert(N <= NN, "node sums");
+    const bool up = (threadIdx.x & bit) != 0;
+#pragma unroll
+    for (int k = 0; k < H; ++k)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const R lo = acc[k][v], hi = H + k < N ? acc[H + k < N ? H + k : 0][v] : R(0);
+            const R got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, bit);
+            acc[k][v] = (up ? hi : lo) + got;
+        }
+    first += up ? H : 0;
+    count = up ? count - H : min(count, H);
+}
+
+// One work item: the cells [cbase, cbase + 32 / G) of a tile.  stg: this block's cp.async
+// staging slots (ST stages x NCM x NT reals); s_item: the item's offsets and tile entry in
+// shared memory; fetch_next() starts the copies of the next item's.  MAT 2 (the adjoint's
 // v_bar scatter) is 3D only.
-template <class R, int D, int NT, int MAT>
-__device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<R> &io, R *stg, int32_t *s_off,
-                                                int k, int cbase, bool &any_escape)
+template <class R, int D, int NT, int MAT, int G, class Next>
+__device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<R> &io, R *stg,
+                                                const int32_t *s_item, int cbase, Next fetch_next,
+                                                bool &any_escape)
 {
     using Gm = Geo<D>;
     constexpr bool ADJ = MAT == 2;
     static_assert(!ADJ || D == 3, "the v_bar scatter is 3D");
     constexpr int NCM = direct_stage_comps<D, MAT>();
     constexpr int NC = ADJ ? 24 : p2g_ncomp<D>(MAT);
-    constexpr int CELLS = direct_cells<D>();
     constexpr int ST = direct_stages<D>();
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t ld = io.ld;
     const R mass = ADJ ? R(0) : P.mass;
-    const int4 t = io.tiles[k];
-    const int sim = (int)(t.x / P.tiles_per_sim);
-    int64_t tl = t.x - (int64_t)sim * P.tiles_per_sim;
+    const int tkey = s_item[kDirectTile];
+    const int first = s_item[kDirectTile + 1];         // the tile's first particle
+    const int sim = tkey / (int)P.tiles_per_sim;
+    int tl = tkey - sim * (int)P.tiles_per_sim;
     int org[3];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        org[a] = (int)(tl % P.n_tiles[a]) * Gm::T;
+        org[a] = tl % P.n_tiles[a] * Gm::T;
         tl /= P.n_tiles[a];
     }
     if constexpr (D == 2) org[2] = 0;
     R4<R> *Asim = io.A + (int64_t)sim * P.nodes_per_sim;
-    const int32_t *pmap = io.posmap + t.y;
-    const int32_t *goff = io.cell_off + (int64_t)t.w * (Gm::TN + 1) + cbase;   // t.w: index in key order
-    // the item's cell offsets, staged once (coalesced) so that the per-cell lookups
-    // below are shared-memory reads (staging the position map as well measured
-    // slower in 3D, 0.125 -> 0.146 ms on the collapse, and no faster in 2D)
-    __syncwarp();
-    for (int i = lane; i <= CELLS; i += 32) s_off[i] = goff[i];
-    __syncwarp();
-    const int32_t *off = s_off - cbase;           // off[c] for the item's cells c in [cbase, cbase + CELLS]
-    auto slot = [&](int q) { return pmap[q]; };
-    const R *St = io.S + t.y;                     // MAT 2: component-major with stride ld
-    const R *S2 = ADJ ? io.src2 + t.y : nullptr;
-    R *const Sv = (ADJ || P.save_S == nullptr) ? nullptr : P.save_S + t.y;
+    // (staging the position map as well measured slower in 3D, 0.125 -> 0.146 ms on the
+    // collapse, and no faster in 2D)
+    const int32_t *pmap = io.posmap + first;
+    const R *St = io.S + first;                   // MAT 2: component-major with stride ld
+    const R *S2 = ADJ ? io.src2 + first : nullptr;
+    R *const Sv = (ADJ || P.save_S == nullptr) ? nullptr : P.save_S + first;
     auto issue = [&](int stage, int32_t pos) {
         R *dst = stg + stage * NCM * NT + tid;
         if constexpr (ADJ) {
@@ -924,83 +933,36 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
 #pragma unroll
             for (int j = 0; j < 21; ++j) cp_async_elem(dst + (3 + j) * NT, S2 + pos + j * ld);
         } else {                                  // the particle state, in blocks of kPB
-            const R *src = io.S + sblock((int64_t)t.y + pos, Lay<D, MAT>::NC);
+            const R *src = io.S + sblock(first + pos, Lay<D, MAT>::NC);
 #pragma unroll
             for (int j = 0; j < NC; ++j) cp_async_elem(dst + j * NT, src + p2g_comp<D, MAT>(j) * kPB);
         }
     };
-    // cursors over this lane's cells cbase + lane + 32 r and their slots
-    struct CurMulti {
-        int c, q, q1, end;
-        __device__ __forceinline__ bool next(const int32_t *o)
-        {
-            ++q;
-            while (q >= q1) {
-                c += 32;
-                if (c >= end) return false;
-                q = o[c];
-                q1 = o[c + 1];
-            }
-            return true;
-        }
-    };
-    // one cell per lane (32-cell items): the cursor walks that cell's particles only
-    struct CurOne {
-        int c, q, q1;
-        __device__ __forceinline__ bool next(const int32_t *) { return ++q < q1; }
-    };
-    using Cur = std::conditional_t<CELLS == 32, CurOne, CurMulti>;
-    Cur pc;
-    if constexpr (CELLS == 32) pc = CurOne{cbase + lane, off[cbase + lane] - 1, off[cbase + lane + 1]};
-    else pc = CurMulti{cbase + lane - 32, 0, 0, cbase + CELLS};
-    Cur cc = pc;
-    bool hp = pc.next(off);
+    constexpr int CPI = 32 / G;
+    const int ci0 = lane % CPI, q_end = s_item[ci0 + 1];
+    const bool any = s_item[ci0] < q_end;         // the lane's cell has particles
+    int pq = s_item[ci0] + lane / CPI, cq = pq;   // slots of the copies and of the sums
+    fetch_next();
 #pragma unroll
     for (int s0 = 0; s0 < ST; ++s0) {
-        if (hp) issue(s0, slot(pc.q));
+        if (pq < q_end) issue(s0, pmap[pq]);
         cp_async_commit();
-        hp = hp && pc.next(off);
+        pq += G;
     }
-    int32_t ppos = hp ? slot(pc.q) : 0;
-    bool hc = cc.next(off);
-    int stage = 0, cur = -1;
-    int bown[D], nb[3];
-    if constexpr (D == 2) nb[2] = 0;
-    unsigned reach = 0u;                          // node tiles (bit dz dy dx) this lane's cells reach
-    CellSums<R, D> acc;
-    auto open_cell = [&](int c) {                 // a new cell: its base, first node, reach; zero sums
-        cur = c;
-        int r = cur;
-        unsigned hi = 0u;
+    int32_t ppos = pq < q_end ? pmap[pq] : 0;
+    int stage = 0;
+    int bown[D];                                  // base cell of the cell's particles
+    {
+        int r = cbase + ci0;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            const int ci = r % Gm::T;
+            bown[a] = org[a] + r % Gm::T - 1;
             r /= Gm::T;
-            bown[a] = org[a] + ci - 1;         // base cell index of the cell's particles
-            nb[a] = org[a] + ci + 1;           // its first stencil node
-            hi |= (ci + 3 >= Gm::T ? 1u : 0u) << a;
         }
-#pragma unroll
-        for (int m = 0; m < (1 << D); ++m)
-            if ((m & ~hi & ((1u << D) - 1u)) == 0u) reach |= 1u << m;
-        acc.zero();
-    };
-    auto close_cell = [&]() {                     // the cell is done: its 3^D node sums to the grid
-        const int sx = P.G_nodes[0], sxy = P.G_nodes[0] * P.G_nodes[1];
-        R4<R> *base = Asim + ((int64_t)nb[2] * P.G_nodes[1] + nb[1]) * sx + nb[0];   // nb[2] = 0 in 2D
-#pragma unroll
-        for (int kk = 0; kk < Gm::STENCIL; ++kk) {
-            R4<R> *node = base + (kk % 3) + ((kk / 3) % 3) * sx + (kk / 9) * sxy;
-            if constexpr (ADJ) red_add4(node, acc.q(kk, 0), acc.q(kk, 1), acc.q(kk, 2), R(0));   // (v_bar, 0)
-            else red_add4(node, acc.m(kk), acc.q(kk, 0), acc.q(kk, 1), acc.q(kk, 2));          // (m, q)
-        }
-    };
-    constexpr bool ONE = CELLS == 32;             // one cell per lane: opened before, closed after the loop
-    if (ONE && hc) open_cell(cc.c);
-    while (hc) {
-        if constexpr (!ONE) {
-            if (cc.c != cur) open_cell(cc.c);
-        }
+    }
+    CellSums<R, D> acc;
+    acc.zero();
+    for (; cq < q_end; cq += G) {
         cp_async_wait<ST - 1>();
         P2GFactors<R, D> f;
         {
@@ -1009,17 +971,17 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
                 adj_scatter_factors<R>(P, [&](int j) { return src[j * NT]; }, f);
             } else {
                 if (Sv != nullptr) {               // the adjoint's copy of this step's state
-                    R *d = Sv + slot(cc.q);
+                    R *d = Sv + pmap[cq];
 #pragma unroll
                     for (int j = 0; j < NC; ++j) d[j * P.n] = src[j * NT];
                 }
                 p2g_factors<R, D, MAT>(P, [&](int j) { return src[j * NT]; }, f);
             }
         }
-        if (hp) issue(stage, ppos);
+        if (pq < q_end) issue(stage, ppos);
         cp_async_commit();
-        hp = hp && pc.next(off);
-        if (hp) ppos = slot(pc.q);
+        pq += G;
+        if (pq < q_end) ppos = pmap[pq];
         bool own = true;
 #pragma unroll
         for (int a = 0; a < D; ++a) own = own && (f.b[a] == bown[a]);
@@ -1032,14 +994,39 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
                              P.node_tiles[1]);
         }
         stage = stage + 1 == ST ? 0 : stage + 1;
-        hc = cc.next(off);
-        if constexpr (!ONE) {
-            if (!hc || cc.c != cur) close_cell();
+    }
+    // the lane's share of the 3^D nodes: all, or nk (at most NODES) of them from k0 on
+    static_assert(G == 1 || G == 4 || G == 8, "lanes per cell");
+    constexpr int H1 = (Gm::STENCIL + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2;
+    constexpr int NODES = G == 1 ? Gm::STENCIL : (G == 4 ? H2 : H3);
+    int k0 = 0, nk = Gm::STENCIL;
+    if constexpr (G > 1) {
+        __syncwarp();
+        share_nodes<Gm::STENCIL>(acc.acc, 16, k0, nk);
+        share_nodes<H1>(acc.acc, 8, k0, nk);
+        if constexpr (G == 8) share_nodes<H2>(acc.acc, 4, k0, nk);
+    }
+    if (any) {                                    // the node sums to the grid; the first node is bown + 2
+        const int sx = P.G_nodes[0], sxy = P.G_nodes[0] * P.G_nodes[1];
+        const int nz = D == 3 ? bown[D - 1] + 2 : 0;
+        R4<R> *base = Asim + ((int64_t)nz * P.G_nodes[1] + bown[1] + 2) * sx + bown[0] + 2;
+#pragma unroll
+        for (int i = 0; i < NODES; ++i) {
+            const int kk = i + k0;
+            if (i >= nk) continue;
+            R4<R> *node = base + (kk % 3) + ((kk / 3) % 3) * sx + (kk / 9) * sxy;
+            if constexpr (ADJ) red_add4(node, acc.q(i, 0), acc.q(i, 1), acc.q(i, 2), R(0));   // (v_bar, 0)
+            else red_add4(node, acc.m(i), acc.q(i, 0), acc.q(i, 1), acc.q(i, 2));           // (m, q)
         }
     }
-    if (ONE && cur >= 0) close_cell();
     cp_async_wait<0>();
-    if constexpr (!ADJ) {                          // node tiles reached by the warp's cells
+    if constexpr (!ADJ) {                          // node tiles (bit dz dy dx) reached by the warp's cells
+        unsigned reach = 0u, hi = 0u;
+#pragma unroll
+        for (int a = 0; a < D; ++a) hi |= (bown[a] - org[a] + 4 >= Gm::T ? 1u : 0u) << a;
+#pragma unroll
+        for (int m = 0; m < (1 << D); ++m)
+            if (any && (m & ~hi & ((1u << D) - 1u)) == 0u) reach |= 1u << m;
         const unsigned wreach = __reduce_or_sync(0xffffffffu, reach);
         if (lane < (1 << D) && ((wreach >> lane) & 1u)) {
             int u[3] = {0, 0, 0};
@@ -1055,29 +1042,65 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
 #ifndef MPM_P2G2_MINB
 #define MPM_P2G2_MINB 4
 #endif
-template <class R, int D, int NT, int MAT>
+// A warp's first item is its own index, later ones come from the cursor, claimed one
+// item ahead; the next item's offsets and tile entry are copied to shared memory while
+// the current one is summed.
+template <class R, int D, int NT, int MAT, int G>
 __global__ void __launch_bounds__(NT, D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB)
     k_p2g_direct(const Params<R> P, const P2GIO<R> io, unsigned long long *__restrict__ escaped_count,
                  int32_t *__restrict__ g2p_cursor)
 {
     using Gm = Geo<D>;
     constexpr int NCM = direct_stage_comps<D, MAT>();
-    constexpr int CELLS = direct_cells<D>();         // cells per work item
-    constexpr int ITEMS = Gm::TN / CELLS;            // work items per tile
+    constexpr int CPI = 32 / G, ITEMS = Gm::TN / CPI;     // cells per item, items per tile
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *stg = reinterpret_cast<R *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31;
-    int32_t *const s_off = reinterpret_cast<int32_t *>(smem_raw + (size_t)direct_stages<D>() * NCM * NT * sizeof(R)) +
-                           (tid >> 5) * kDirectOffPad;
-    const int n_items = *io.n_tiles * ITEMS;
+    int32_t *const s_items = reinterpret_cast<int32_t *>(smem_raw + (size_t)direct_stages<D>() * NCM * NT * sizeof(R)) +
+                             (tid >> 5) * 2 * kDirectItemInts;
+    __shared__ int s_n;                              // number of items
+    if (tid == 0) s_n = *io.n_tiles * ITEMS;
+    __syncthreads();
     bool any_escape = false;
-    for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(io.cursor, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item >= n_items) break;
+    auto fetch = [&](int item, int32_t *s) {         // copies started here, complete after a wait for all groups
         const int k = item / ITEMS;
-        p2g_direct_item<R, D, NT, MAT>(P, io, stg, s_off, k, (item - k * ITEMS) * CELLS, any_escape);
+        const int32_t *goff = io.cell_off + (int64_t)k * (Gm::TN + 1) + (item - k * ITEMS) * CPI;
+        if (G == 1 || lane < CPI) cp_async_elem(s + lane, goff + lane);
+        if (lane == 0) cp_async_elem(s + CPI, goff + CPI);
+        if (lane < 2) cp_async_elem(s + kDirectTile + lane, reinterpret_cast<const int32_t *>(io.tiles + k) + lane);
+        if (lane == 0) s[kDirectTile + 2] = item;
+    };
+    auto claim = [&]() {
+        const int warps = (int)gridDim.x * (NT / 32);
+        return lane == 0 && s_n > warps ? warps + atomicAdd(io.cursor, 1) : s_n;
+    };
+    int slot = 0, ahead = s_n;                       // ahead (lane 0): the item after the current one
+    {
+        const int item = blockIdx.x * (NT / 32) + (tid >> 5);
+        if (item < s_n) {
+            fetch(item, s_items);
+            cp_async_commit();
+            ahead = claim();
+            cp_async_wait<0>();
+        } else {
+            slot = -1;
+        }
+    }
+    __syncwarp();
+    while (slot >= 0) {
+        const int next = __shfl_sync(0xffffffffu, ahead, 0);
+        const bool more = next < s_n;
+        const int32_t *s = s_items + slot * kDirectItemInts;
+        slot = more ? slot ^ 1 : -1;
+        p2g_direct_item<R, D, NT, MAT, G>(
+            P, io, stg, s, s[kDirectTile + 2] % ITEMS * CPI,
+            [&]() {
+                if (!more) return;
+                fetch(next, s_items + slot * kDirectItemInts);
+                ahead = claim();
+            },
+            any_escape);
+        __syncwarp();
     }
     if (escaped_count != nullptr) {
         const unsigned ball = __ballot_sync(0xffffffffu, any_escape);
@@ -1997,6 +2020,17 @@ Params<R> make_params(const HostParams &h, const DevState &ds)
     return P;
 }
 
+// Whether the cell-ordered P2G gives a cell's particles kShareLanes lanes: the halving
+// exchanges pay while the cells are too few for the chip's lanes (32 steps without | with:
+// 2D, 8,192 particles 605 | 412 us, 294,912: 1480 | 1446, 589,824: 1639 | 1871; 3D, 50,560:
+// 1259 | 961, 86,592: 1372 | 1369, 169,680: 1491 | 1603).
+template <int D> constexpr int kShareLanes = D == 3 ? 4 : 8;
+template <int D> inline bool p2g_share(int64_t n, int num_sms)
+{
+    const int64_t lanes = (int64_t)num_sms * (D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB) * 128;
+    return n <= (D == 3 ? 1 : 4) * lanes;
+}
+
 inline int grid_blocks(int64_t n, int threads, int num_sms, int per_sm = 16)
 {
     int64_t b = (n + threads - 1) / threads;
@@ -2026,38 +2060,45 @@ template <class R, int D> struct Launch {
     static constexpr bool kReg = (sizeof(R) == 4) || (D == 2);
     static constexpr int kP2GThreads = (D == 3 && kReg) ? 128 : 256;
     static size_t p2g_smem() { return p2g_smem_bytes<R, D, kP2GThreads>(); }
+    // the cell-ordered P2G with G lanes per cell
+    template <int MAT, int G> static void p2g_direct_launch(const HostParams &h, DevState &ds)
+    {
+        auto P = make_params<R>(h, ds);
+        constexpr int NT = 128;
+        constexpr size_t smem = p2g_direct_smem<R, D, NT, MAT>();
+        static_assert(smem <= 48 * 1024, "k_p2g_direct shared memory above the default limit");
+        // persistent: as many blocks as fit on the GPU at once (3D: the launch
+        // bound's MPM_P2G_MINB per SM; 2D: more, its accumulators are 27 values)
+        static int per_sm = 0;
+        if (per_sm == 0) {
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2g_direct<R, D, NT, MAT, G>, NT, smem) !=
+                    cudaSuccess ||
+                per_sm < 1)
+                per_sm = MPM_P2G_MINB;
+        }
+        const int nb = ds.num_sms * per_sm;
+        // tiles in key order (claiming them largest first, as G2P does, measured slower)
+        P2GIO<R> io{(const R *)ds.S, nullptr, h.npad, ds.tiles, ds.counters + 1, ds.counters + 2, ds.posmap,
+                    ds.cell_off, (R4<R> *)ds.A, ds.flags};
+        k_p2g_direct<R, D, NT, MAT, G><<<nb, NT, smem, ds.stream>>>(P, io, ds.escaped, ds.counters + 3);
+        if (h.transfer == 3) {                       // FLIP: the momenta without forces, for v_i^n
+            auto P2 = P;
+            P2.no_force = 1;
+            P2.save_S = nullptr;
+            cudaMemsetAsync(ds.counters + 2, 0, sizeof(int32_t), ds.stream);
+            io.A = (R4<R> *)ds.A2;
+            k_p2g_direct<R, D, NT, MAT, G><<<nb, NT, smem, ds.stream>>>(P2, io, ds.escaped, ds.counters + 3);
+        }
+    }
     // one instantiation per material (the staged component count is a compile-time constant)
     template <int MAT> static void p2g_launch(const HostParams &h, DevState &ds)
     {
-        auto P = make_params<R>(h, ds);
         if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) {
-            constexpr int NT = 128;
-            constexpr size_t smem = p2g_direct_smem<R, D, NT, MAT>();
-            static_assert(smem <= 48 * 1024, "k_p2g_direct shared memory above the default limit");
-            // persistent: as many blocks as fit on the GPU at once (3D: the launch
-            // bound's MPM_P2G_MINB per SM; 2D: more, its accumulators are 27 values)
-            static int per_sm = 0;
-            if (per_sm == 0) {
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2g_direct<R, D, NT, MAT>, NT, smem) !=
-                        cudaSuccess ||
-                    per_sm < 1)
-                    per_sm = MPM_P2G_MINB;
-            }
-            const int nb = ds.num_sms * per_sm;
-            // tiles in key order (claiming them largest first, as G2P does, measured slower)
-            P2GIO<R> io{(const R *)ds.S, nullptr, h.npad, ds.tiles, ds.counters + 1, ds.counters + 2, ds.posmap,
-                        ds.cell_off, (R4<R> *)ds.A, ds.flags};
-            k_p2g_direct<R, D, NT, MAT><<<nb, NT, smem, ds.stream>>>(P, io, ds.escaped, ds.counters + 3);
-            if (h.transfer == 3) {                   // FLIP: the momenta without forces, for v_i^n
-                auto P2 = P;
-                P2.no_force = 1;
-                P2.save_S = nullptr;
-                cudaMemsetAsync(ds.counters + 2, 0, sizeof(int32_t), ds.stream);
-                io.A = (R4<R> *)ds.A2;
-                k_p2g_direct<R, D, NT, MAT><<<nb, NT, smem, ds.stream>>>(P2, io, ds.escaped, ds.counters + 3);
-            }
+            if (p2g_share<D>(h.n, ds.num_sms)) p2g_direct_launch<MAT, kShareLanes<D>>(h, ds);
+            else p2g_direct_launch<MAT, 1>(h, ds);
             return;
         }
+        auto P = make_params<R>(h, ds);
         const size_t smem = p2g_smem();
         static bool attr = false;
         if (!attr) {
