@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
                               const R *__restrict__ lam_in, R *__restrict__ lam_out, R4<R> *__restrict__ GVB)
 {
     const int64_t n = P.n;
+    pdl_wait();
     constexpr int JC = 2 * D, JR = 2 * D + D * D;
     const R cscale = R(4) * P.inv_dx;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
@@ -661,6 +662,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
         for (int a = 0; a < D; ++a) lam_out[a * n + p] = xb[a];
         lam_out[JR * n + p] = rhob;
     }
+    pdl_release();
 }
 
 // Adjoint of the grid update per node: GVB (adjoint of v) -> GAB (adjoint of m, P)
@@ -674,6 +676,7 @@ __global__ void __launch_bounds__(256) k_adj_grid_bwd(const Params<R> P, const R
                                                       int32_t *__restrict__ scatter_cursor)
 {
     using Gm = Geo<D>;
+    pdl_wait();
     if (scatter_cursor != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *scatter_cursor = 0;
     const int n_list = GL[0];
     for (int li = blockIdx.x; li < n_list; li += gridDim.x) {
@@ -723,6 +726,7 @@ __global__ void __launch_bounds__(256) k_adj_grid_bwd(const Params<R> P, const R
         GAB[i] = R4<R>{mb, ob[0] * inv_m, ob[1] * inv_m, D == 3 ? ob[2] * inv_m : R(0)};
     }
     }
+    pdl_release();
 }
 
 // Adjoint of P2G for one particle; completes lam_out (adjoint of S^t).
@@ -731,6 +735,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
                               R *__restrict__ lam_out)
 {
     const int64_t n = P.n;
+    pdl_wait();
     constexpr int JV = D, JC = 2 * D, JR = 2 * D + D * D;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         R x[D], v[D], C[D * D];
@@ -864,6 +869,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
         for (int q = 0; q < D * D; ++q) lam_out[(JC + q) * n + p] = Cb[q];
         lam_out[JR * n + p] += sb * dsdrho;
     }
+    pdl_release();
 }
 
 // ------------------------------------------------------------------ 3D reverse kernels in separable form
@@ -1152,6 +1158,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3_MINB : 1)
 {
     constexpr int D = 3, JC = 2 * D, JR = 2 * D + D * D;
     const int64_t n = P.n;
+    pdl_wait();
     const R cscale = R(4) * P.inv_dx;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         R x[D];
@@ -1268,6 +1275,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3_MINB : 1)
         for (int a = 0; a < D; ++a) lam_out[a * n + p] = xb[a];
         lam_out[JR * n + p] = rb1 / den;
     }
+    pdl_release();
 }
 
 // 3D adjoint of P2G (same outputs as k_adj_p2g_bwd) from stencil moments of the
@@ -1279,6 +1287,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3P_MINB : 1)
 {
     constexpr int D = 3, JV = D, JC = 2 * D, JR = 2 * D + D * D;
     const int64_t n = P.n;
+    pdl_wait();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         R x[D], v[D], C[D * D];
 #pragma unroll
@@ -1371,6 +1380,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3P_MINB : 1)
             lam_out[JR * n + p] += sb * dsdrho;
         }
     }
+    pdl_release();
 }
 
 // ------------------------------------------------------------------ launchers
@@ -1456,8 +1466,8 @@ template <class R, int D> struct AdjLaunch {
             if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) split = a.coef != nullptr && a.tiles != nullptr;
             if (split) {
                 if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) {
-                    k_adj_g2p_bwd3<R, true><<<pblocks(h, ds), 256, 0, ds.stream>>>(
-                        P, (const R *)st, (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB,
+                    launch_after(
+                        k_adj_g2p_bwd3<R, true>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB,
                         (R *)a.coef);
                     constexpr int NT = 128;
                     constexpr size_t smem = p2g_direct_smem<R, 3, NT, 2>();
@@ -1466,29 +1476,29 @@ template <class R, int D> struct AdjLaunch {
                                 a.cell_off, (R4<R> *)a.GVB, nullptr};
                     const int nb = ds.num_sms * MPM_P2G_MINB;
                     if (p2g_share<3>(h.n, ds.num_sms))
-                        k_p2g_direct<R, 3, NT, 2, kShareLanes<3>><<<nb, NT, smem, ds.stream>>>(P, io, nullptr, nullptr);
+                        launch_after(k_p2g_direct<R, 3, NT, 2, kShareLanes<3>>, nb, NT, smem, ds.stream, P, io, nullptr, nullptr);
                     else
-                        k_p2g_direct<R, 3, NT, 2, 1><<<nb, NT, smem, ds.stream>>>(P, io, nullptr, nullptr);
+                        launch_after(k_p2g_direct<R, 3, NT, 2, 1>, nb, NT, smem, ds.stream, P, io, nullptr, nullptr);
                 }
             } else {
-                k_adj_g2p_bwd3<R, false><<<pblocks(h, ds), 256, 0, ds.stream>>>(
-                    P, (const R *)st, (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB, nullptr);
+                launch_after(
+                    k_adj_g2p_bwd3<R, false>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB, nullptr);
             }
         } else {
-            k_adj_g2p_bwd<R, D><<<pblocks(h, ds), 256, 0, ds.stream>>>(P, (const R *)st, (const R4<R> *)GV,
+            launch_after(k_adj_g2p_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)GV,
                                                                          (const R *)lam_in, (R *)lam_out,
                                                                          (R4<R> *)a.GVB);
         }
         int64_t nbg = h.node_tiles_per_sim;             // blocks stride the saved tile list
         if (nbg > (int64_t)ds.num_sms * 8) nbg = (int64_t)ds.num_sms * 8;
-        k_adj_grid_bwd<R, D><<<(unsigned)nbg, 256, 0, ds.stream>>>(P, (const R4<R> *)GA, (R4<R> *)a.GVB,
+        launch_after(k_adj_grid_bwd<R, D>, (unsigned)nbg, 256, 0, ds.stream, P, (const R4<R> *)GA, (R4<R> *)a.GVB,
                                                                    (R4<R> *)a.GAB, GL, mub,
                                                                    split ? a.cursor : nullptr);
         if constexpr (D == 3 && MPM_ADJ_SEPARABLE)
-            k_adj_p2g_bwd3<R><<<pblocks(h, ds), 256, 0, ds.stream>>>(P, (const R *)st, (const R4<R> *)a.GAB,
+            launch_after(k_adj_p2g_bwd3<R>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)a.GAB,
                                                                    (R *)lam_out);
         else
-            k_adj_p2g_bwd<R, D><<<pblocks(h, ds), 256, 0, ds.stream>>>(P, (const R *)st, (const R4<R> *)a.GAB,
+            launch_after(k_adj_p2g_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)a.GAB,
                                                                          (R *)lam_out);
     }
 };

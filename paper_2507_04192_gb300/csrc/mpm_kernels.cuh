@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(NT, (D == 3 && REG) ? MPM_P2G_MINB : 1)
     __shared__ int s_slot;
     const int n_tiles = counters[1];
     const int tid = threadIdx.x;
+    pdl_wait();
     for (;;) {
         const int k = next_tile(&counters[2], n_tiles, &s_slot);
         if (k < 0) break;
@@ -697,6 +698,7 @@ __global__ void __launch_bounds__(NT, (D == 3 && REG) ? MPM_P2G_MINB : 1)
                            (int64_t)sim * P.node_tiles_per_sim + lin3<D>(u, P.node_tiles));
         }
     }
+    pdl_release();
     if (threadIdx.x == 0) counters[3] = 0;         // G2P cursor for the next kernel (G2P follows)
 }
 
@@ -1077,14 +1079,12 @@ __global__ void __launch_bounds__(NT, D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB)
     int slot = 0, ahead = s_n;                       // ahead (lane 0): the item after the current one
     {
         const int item = blockIdx.x * (NT / 32) + (tid >> 5);
-        if (item < s_n) {
-            fetch(item, s_items);
-            cp_async_commit();
-            ahead = claim();
-            cp_async_wait<0>();
-        } else {
-            slot = -1;
-        }
+        if (item < s_n) fetch(item, s_items);        // the sort's tables: complete before the last kernel began
+        cp_async_commit();
+        pdl_enter();
+        if (item < s_n) ahead = claim();
+        else slot = -1;
+        cp_async_wait<0>();
     }
     __syncwarp();
     while (slot >= 0) {
@@ -1159,6 +1159,7 @@ __global__ void __launch_bounds__(256) k_grid(const Params<R> P, R4<R> *__restri
                                               const int32_t *__restrict__ count)
 {
     using Gm = Geo<D>;
+    pdl_wait();
     const int n_list = *count;
     if (saveL != nullptr && blockIdx.x == 0 && threadIdx.x == 0) saveL[0] = n_list;
     // conservation sums (P.diag set): mass, momentum (q + dt f), non-finite values, sum of |q|
@@ -1245,6 +1246,7 @@ __global__ void __launch_bounds__(256) k_grid(const Params<R> P, R4<R> *__restri
     }
     if (threadIdx.x == 0) flags[ut] = 0u;
     }
+    pdl_release();
     if (P.diag != nullptr) {
         constexpr int slots[6] = {kDiagGridMass, kDiagGridMom, kDiagGridMom + 1, kDiagGridMom + 2, kDiagGridNonFinite,
                                   kDiagGridAbsMom};
@@ -1700,16 +1702,15 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
     R *const bufs = reinterpret_cast<R *>(base + 2 * L::win_bytes) + (size_t)warp * 2 * L::blk_elems;
     const bool withhold = (P.debug & kDebugWithholdWindowCopy) != 0;
     const int n_items = counters[6];
+    const int4 none = make_int4(0, 0, 0, 0), first = (int)blockIdx.x < n_items ? items[blockIdx.x] : none;
     int claim = n_items;                           // thread 0: the item after the published ones
     auto take = [&]() { return n_items > (int)gridDim.x ? (int)gridDim.x + atomicAdd(&counters[3], 1) : n_items; };
-    auto publish = [&](int slot, int id) {         // thread 0: item id and its window to a slot (count 0: no more)
-        if (id >= n_items) {
-            s_item[slot] = make_int4(0, 0, 0, 0);
+    auto publish = [&](int slot, int4 t) {         // thread 0: an item and its window to a slot (count 0: no more)
+        s_item[slot] = t;
+        if (t.w == 0) {
             mbar_arrive(&full[slot]);
             return;
         }
-        const int4 t = items[id];
-        s_item[slot] = t;
         if (withhold) return;
         const int org[3] = {(t.y & 1023) * Gm::T, ((t.y >> 10) & 1023) * Gm::T, (t.y >> 20) * Gm::T};
         fence_proxy_async_smem();
@@ -1726,9 +1727,28 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
         fence_mbar_init();
     }
     __syncthreads();
+    // this warp's particle blocks b of item t: b0, b0 + 8, ... below b1
+    auto stage = [&](int b, int d) {
+        if (lane == 0) {
+            fence_proxy_async_smem();
+            mbar_expect_tx(&blk[warp][d], (uint32_t)(L::blk_elems * sizeof(R)));
+            bulk_g2s(bufs + d * L::blk_elems, S + (int64_t)b * Ly::NC * kPB, (uint32_t)(L::blk_elems * sizeof(R)),
+                     &blk[warp][d]);
+        }
+    };
+    auto stage_first = [&](const int4 &t) {
+        const int b = t.z / kPB + warp, b1 = (t.z + t.w + kPB - 1) / kPB;
+        if (t.w > 0 && b < b1) stage(b, 0);
+        if (t.w > 0 && b + NW < b1) stage(b + NW, 1);
+    };
+    // the first item's particles: unchanged since the last G2P, which was complete
+    // before the grid update before this kernel let it start
+    stage_first(first);
+    pdl_wait();
     if (tid == 0) {
-        publish(0, blockIdx.x);
-        publish(1, take());
+        publish(0, first);
+        const int second = take();
+        publish(1, second < n_items ? items[second] : none);
         claim = take();
     }
     bool bad = false, timed_out = false;
@@ -1739,9 +1759,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
         timed_out = !mbar_wait_bounded(&full[slot], ph);
         if (__any_sync(0xffffffffu, timed_out)) {
             timed_out = true;
-            if (!withhold) {                       // the windows in flight land before the block leaves
+            if (!withhold) {                       // the copies in flight land before the block leaves
                 mbar_wait_bounded(&full[slot], ph);
                 mbar_wait_bounded(&full[slot ^ 1], (uint32_t)((i + 1) >> 1) & 1u);
+            }
+            if (i == 0) {
+                const int b = first.z / kPB + warp, b1 = (first.z + first.w + kPB - 1) / kPB;
+                if (first.w > 0 && b < b1) mbar_wait_bounded(&blk[warp][0], 0u);
+                if (first.w > 0 && b + NW < b1) mbar_wait_bounded(&blk[warp][1], 0u);
             }
             break;
         }
@@ -1750,17 +1775,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
         const int org[3] = {(t.y & 1023) * Gm::T, ((t.y >> 10) & 1023) * Gm::T, (t.y >> 20) * Gm::T};
         const R4<R> *Vw = wins + slot * L::win_elems;
         const int b1 = (t.z + t.w + kPB - 1) / kPB;            // particle blocks [t.z / kPB, b1)
-        auto stage = [&](int b, int d) {
-            if (lane == 0) {
-                fence_proxy_async_smem();
-                mbar_expect_tx(&blk[warp][d], (uint32_t)(L::blk_elems * sizeof(R)));
-                bulk_g2s(bufs + d * L::blk_elems, S + (int64_t)b * Ly::NC * kPB, (uint32_t)(L::blk_elems * sizeof(R)),
-                         &blk[warp][d]);
-            }
-        };
         int b = t.z / kPB + warp, d = 0;
-        if (b < b1) stage(b, 0);
-        if (b + NW < b1) stage(b + NW, 1);
+        if (i > 0) stage_first(t);
         for (; b < b1; b += NW, d ^= 1) {
             if (!mbar_wait_bounded(&blk[warp][d], (phases >> d) & 1u)) timed_out = true;
             phases ^= 1u << d;
@@ -1778,7 +1794,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
         if (lane == 0) mbar_arrive(&empty[slot]);
         if (tid == 0) {                            // the next item but one, once every warp has left this window
             if (!timed_out && mbar_wait_bounded(&empty[slot], ph)) {
-                publish(slot, claim);
+                publish(slot, claim < n_items ? items[claim] : none);
                 if (claim < n_items) claim = take();
             } else {
                 timed_out = true;
@@ -1790,6 +1806,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_G2P_MINB : 1)
             break;
         }
     }
+    pdl_release();
     if (timed_out && lane == 0) atomicOr(status, (int32_t)kStatusTimeout);
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, (int32_t)kStatusNaN);
     if (tid == 0) {
@@ -2080,14 +2097,14 @@ template <class R, int D> struct Launch {
         // tiles in key order (claiming them largest first, as G2P does, measured slower)
         P2GIO<R> io{(const R *)ds.S, nullptr, h.npad, ds.tiles, ds.counters + 1, ds.counters + 2, ds.posmap,
                     ds.cell_off, (R4<R> *)ds.A, ds.flags};
-        k_p2g_direct<R, D, NT, MAT, G><<<nb, NT, smem, ds.stream>>>(P, io, ds.escaped, ds.counters + 3);
+        launch_after(k_p2g_direct<R, D, NT, MAT, G>, nb, NT, smem, ds.stream, P, io, ds.escaped, ds.counters + 3);
         if (h.transfer == 3) {                       // FLIP: the momenta without forces, for v_i^n
             auto P2 = P;
             P2.no_force = 1;
             P2.save_S = nullptr;
             cudaMemsetAsync(ds.counters + 2, 0, sizeof(int32_t), ds.stream);
             io.A = (R4<R> *)ds.A2;
-            k_p2g_direct<R, D, NT, MAT, G><<<nb, NT, smem, ds.stream>>>(P2, io, ds.escaped, ds.counters + 3);
+            launch_after(k_p2g_direct<R, D, NT, MAT, G>, nb, NT, smem, ds.stream, P2, io, ds.escaped, ds.counters + 3);
         }
     }
     // one instantiation per material (the staged component count is a compile-time constant)
@@ -2110,15 +2127,15 @@ template <class R, int D> struct Launch {
         const int64_t cap = (int64_t)ds.num_sms * (kP2GThreads == 128 ? MPM_P2G_MINB : 2);
         if (nb > cap) nb = cap;
         if (nb < 1) nb = 1;
-        k_p2g<R, D, kReg, kP2GThreads, MAT><<<(int)nb, kP2GThreads, smem, ds.stream>>>(
-            P, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A, ds.flags, ds.escaped);
+        launch_after(
+            k_p2g<R, D, kReg, kP2GThreads, MAT>, (int)nb, kP2GThreads, smem, ds.stream, P, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A, ds.flags, ds.escaped);
         if (h.transfer == 3) {                       // FLIP: the momenta without forces, for v_i^n
             auto P2 = P;
             P2.no_force = 1;
             P2.save_S = nullptr;
             cudaMemsetAsync(ds.counters + 2, 0, sizeof(int32_t), ds.stream);
-            k_p2g<R, D, kReg, kP2GThreads, MAT><<<(int)nb, kP2GThreads, smem, ds.stream>>>(
-                P2, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A2, ds.flags,
+            launch_after(
+                k_p2g<R, D, kReg, kP2GThreads, MAT>, (int)nb, kP2GThreads, smem, ds.stream, P2, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A2, ds.flags,
                 ds.escaped);
         }
     }
@@ -2132,7 +2149,7 @@ template <class R, int D> struct Launch {
         auto P = make_params<R>(h, ds);
         int64_t nb = h.batch * h.node_tiles_per_sim;        // blocks walk the touched-tile list
         if (nb > (int64_t)ds.num_sms * 8) nb = (int64_t)ds.num_sms * 8;
-        k_grid<R, D><<<(unsigned)nb, 256, 0, ds.stream>>>(P, (R4<R> *)ds.A, (R4<R> *)ds.V, ds.flags,
+        launch_after(k_grid<R, D>, (unsigned)nb, 256, 0, ds.stream, P, (R4<R> *)ds.A, (R4<R> *)ds.V, ds.flags,
                                                            (R4<R> *)ds.save_A, (R4<R> *)ds.save_V,
                                                            ds.save_L, (R4<R> *)ds.A2, (R4<R> *)ds.V2,
                                                            ds.node_list, ds.counters + 4);
@@ -2160,8 +2177,8 @@ template <class R, int D> struct Launch {
         const int64_t cap = (int64_t)ds.num_sms * per_sm;
         if (nb > cap) nb = cap;
         if (nb < 1) nb = 1;
-        k_g2p<R, D, GENERIC, MAT><<<(int)nb, G2PSmem<R, D, MAT>::NT, smem, ds.stream>>>(
-            P, ds.tmap_V, (R *)ds.S, (const R4<R> *)ds.V, ds.items, ds.counters, ds.status,
+        launch_after(
+            k_g2p<R, D, GENERIC, MAT>, (int)nb, G2PSmem<R, D, MAT>::NT, smem, ds.stream, P, ds.tmap_V, (R *)ds.S, (const R4<R> *)ds.V, ds.items, ds.counters, ds.status,
             (const R4<R> *)ds.V2);
     }
     static void g2p(const HostParams &h, DevState &ds)

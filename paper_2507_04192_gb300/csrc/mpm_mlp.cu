@@ -23,6 +23,7 @@ namespace {
 
 __global__ void k_f32_to_bf16(const float *__restrict__ in, __nv_bfloat16 *__restrict__ out, int64_t n)
 {
+    pdl_enter();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = __float2bfloat16_rn(in[i]);
 }
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(256) k_prepare_input(const float *__restrict__
 {
     __shared__ __nv_bfloat16 tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    pdl_enter();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *loss = 0.0;
     for (int j = ty; j < 32; j += 8) {
         const int r = r0 + j, c = c0 + tx;
@@ -81,6 +83,7 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
     __shared__ __nv_bfloat16 tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int64_t n = (int64_t)rows * cols;
+    pdl_enter();
     double acc = 0.0;
     for (int j = ty; j < 32; j += 8) {
         const int r = r0 + j, c = c0 + tx;
@@ -153,6 +156,7 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
     __shared__ float rows[256][32];
     __shared__ float tile[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, blk = blockIdx.x;
+    pdl_enter();
     if (blk == 0 && threadIdx.x == 0 && s.loss_out != nullptr) *s.loss_out = *s.loss;
     int l = 0;
     if (blk < s.n_bias) {
@@ -356,7 +360,7 @@ int backward_update(mpm_mlp *m, int B, double lr, int update, double *loss_out)
         s.layer[l].tile0 = blocks;
         blocks += ((m->w[l + 1] + 31) / 32) * ((m->w[l] + 31) / 32);
     }
-    k_step_end<<<blocks, 256, 0, m->stream>>>(s);
+    launch_after(k_step_end, blocks, 256, 0, m->stream, s);
     return MPM_OK;
 }
 
@@ -370,11 +374,11 @@ int train_queue(mpm_mlp *m, int B, const float *x, const float *src, double lr, 
     const float *xd = on_device(m, x, m->X0f, (int64_t)B * nin, device);
     const float *sd = on_device(m, src, m->T, (int64_t)B * nout, device);
     if (!xd || !sd) return MPM_ECUDA;
-    k_prepare_input<<<dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream>>>(xd, m->X[0], m->XT[0], B, nin, m->loss);
+    launch_after(k_prepare_input, dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream, xd, m->X[0], m->XT[0], B, nin, m->loss);
     int rc = forward(m, B, true);
     if (rc != MPM_OK) return rc;
-    k_output_grad<<<dim3((nout + 31) / 32, (B + 31) / 32), 256, 0, m->stream>>>(
-        m->Y, sd, m->Z[L - 1], m->dZ[L - 1], m->dZb[L - 1], m->dZbT[L - 1], B, nout, m->lo, m->hi,
+    launch_after(
+        k_output_grad, dim3((nout + 31) / 32, (B + 31) / 32), 256, 0, m->stream, m->Y, sd, m->Z[L - 1], m->dZ[L - 1], m->dZb[L - 1], m->dZbT[L - 1], B, nout, m->lo, m->hi,
         m->out_act == MPM_OUT_LINEAR, with_loss ? m->loss : nullptr);
     rc = backward_update(m, B, lr, update, loss_out);
     return rc != MPM_OK ? rc : check(m);
@@ -524,7 +528,7 @@ int mpm_mlp_infer(mpm_mlp *m, int batch, const float *x, float *y, int device_pt
     const int64_t nx = (int64_t)batch * m->w[0];
     const float *xd = on_device(m, x, m->X0f, nx, device_ptrs != 0);
     if (!xd) return MPM_ECUDA;
-    k_f32_to_bf16<<<blocks_for(nx), 256, 0, m->stream>>>(xd, m->X[0], nx);
+    launch_after(k_f32_to_bf16, blocks_for(nx), 256, 0, m->stream, xd, m->X[0], nx);
     int rc = forward(m, batch, false);
     if (rc == MPM_OK) rc = check(m);
     if (rc != MPM_OK) return rc;

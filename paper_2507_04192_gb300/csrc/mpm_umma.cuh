@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
+    pdl_enter();
 
     if (tid == 0) {                                        // producer
         for (int kc = 0; kc < nk; ++kc) {
@@ -392,6 +393,7 @@ __global__ void __launch_bounds__(kUmmaPersistThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
+    pdl_enter();
 
     if (warp == 0) {                                     // producer
         if (lane == 0) {
@@ -592,7 +594,7 @@ inline cudaError_t umma_launch(const UmmaGemm *g, int n, int32_t *status, cudaSt
         blocks += j.tiles;
     }
     if (n == 1) jobs.j[1] = jobs.j[0];
-    k_umma_gemm_tma<NT, STAGES><<<blocks, kUmmaThreads, smem, stream>>>(jobs, status);
+    launch_after(k_umma_gemm_tma<NT, STAGES>, blocks, kUmmaThreads, smem, stream, jobs, status);
     return cudaGetLastError();
 }
 
@@ -632,8 +634,8 @@ inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, in
             attr = true;
         }
         const int tiles = ((M + kUmmaM - 1) / kUmmaM) * ((N + 255) / 256);
-        k_umma_gemm_persist<MPM_UMMA_WIDE_STAGES><<<std::min(sms, tiles), kUmmaPersistThreads, smem, stream>>>(
-            M, N, K, tmA, tmB, C, ldc, epi, status);
+        launch_after(
+            k_umma_gemm_persist<MPM_UMMA_WIDE_STAGES>, std::min(sms, tiles), kUmmaPersistThreads, smem, stream, M, N, K, tmA, tmB, C, ldc, epi, status);
         return cudaGetLastError();
     }
     const UmmaGemm g{M, N, K, A, lda, B, ldb, C, ldc, epi};
