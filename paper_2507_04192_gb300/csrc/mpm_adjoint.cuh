@@ -1463,9 +1463,9 @@ template <class R, int D> struct AdjLaunch {
         auto P = make_params<R>(h, ds);
         bool split = false;
         if constexpr (D == 3 && MPM_ADJ_SEPARABLE) {
-            if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) split = a.coef != nullptr && a.tiles != nullptr;
+            if constexpr (sizeof(R) == 4) split = a.coef != nullptr && a.tiles != nullptr;
             if (split) {
-                if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) {
+                if constexpr (sizeof(R) == 4) {
                     launch_after(
                         k_adj_g2p_bwd3<R, true>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB,
                         (R *)a.coef);

@@ -381,11 +381,11 @@ __device__ __forceinline__ void p2g_node(const P2GFactors<R, D> &f, R mp, int k0
     }
 }
 
-// Sum one particle's contributions into per-cell register accumulators (its
-// base is the cell's base).  Products shared by the three nodes of a z-column
+// Sum one particle's contributions into per-cell accumulators acc(k, v) (its base is
+// the cell's base).  Products shared by the three nodes of a z-column
 // are formed once per (k0, k1).
-template <class R, int D>
-__device__ __forceinline__ void p2g_accumulate(const P2GFactors<R, D> &f, R mp, R (&acc)[Geo<D>::STENCIL][D + 1])
+template <class R, int D, class Acc>
+__device__ __forceinline__ void p2g_accumulate(const P2GFactors<R, D> &f, R mp, Acc acc)
 {
     if constexpr (D == 2) {
 #pragma unroll
@@ -393,10 +393,10 @@ __device__ __forceinline__ void p2g_accumulate(const P2GFactors<R, D> &f, R mp, 
 #pragma unroll
             for (int k0 = 0; k0 < 3; ++k0) {
                 const int k = k1 * 3 + k0;
-                acc[k][0] = fma(mp * f.w[0][k0], f.w[1][k1], acc[k][0]);
+                acc(k, 0) = fma(mp * f.w[0][k0], f.w[1][k1], acc(k, 0));
 #pragma unroll
                 for (int a = 0; a < D; ++a)           // two chained fused multiply-adds per value
-                    acc[k][1 + a] = fma(f.E[a][0][k0], f.w[1][k1], fma(f.w[0][k0], f.E[a][1][k1], acc[k][1 + a]));
+                    acc(k, 1 + a) = fma(f.E[a][0][k0], f.w[1][k1], fma(f.w[0][k0], f.E[a][1][k1], acc(k, 1 + a)));
             }
     } else {
 #pragma unroll
@@ -411,30 +411,13 @@ __device__ __forceinline__ void p2g_accumulate(const P2GFactors<R, D> &f, R mp, 
 #pragma unroll
                 for (int k2 = 0; k2 < 3; ++k2) {
                     const int k = (k2 * 3 + k1) * 3 + k0;
-                    acc[k][0] = fma(mwxy, f.w[2][k2], acc[k][0]);
+                    acc(k, 0) = fma(mwxy, f.w[2][k2], acc(k, 0));
 #pragma unroll
                     for (int a = 0; a < D; ++a)
-                        acc[k][1 + a] = fma(f.w[2][k2], Tm[a], fma(wxy, f.E[a][2][k2], acc[k][1 + a]));
+                        acc(k, 1 + a) = fma(f.w[2][k2], Tm[a], fma(wxy, f.E[a][2][k2], acc(k, 1 + a)));
                 }
             }
     }
-}
-
-// Byte offset of the P2G per-thread staging slots in dynamic shared memory
-// (after the window and the cell offsets, 16-byte aligned) and the total size.
-template <class R, int D> __host__ __device__ constexpr size_t p2g_stage_offset()
-{
-    return ((size_t)(D + 1) * Geo<D>::WN * sizeof(R) + (Geo<D>::TN + 1) * sizeof(int32_t) + 15) & ~size_t(15);
-}
-// Particles in flight per P2G thread (cp.async stages of its staging slots; 3
-// measured slower than 2 on the 3D collapse).
-#ifndef MPM_P2G_STAGES
-#define MPM_P2G_STAGES 2
-#endif
-
-template <class R, int D, int NT> __host__ __device__ constexpr size_t p2g_smem_bytes()
-{
-    return p2g_stage_offset<R, D>() + (size_t)MPM_P2G_STAGES * p2g_ncomp<D>(1) * NT * sizeof(R);
 }
 
 template <int D> __device__ __forceinline__ int win_index(const int l[D], int k0, int k1, int k2)
@@ -451,55 +434,6 @@ __device__ __forceinline__ void mark_node_tile(uint32_t *flags, int32_t *list, i
     if (flags[g] == 0u && atomicExch(&flags[g], 1u) == 0u) list[atomicAdd(count, 1)] = (int32_t)g;
 }
 
-// Scatter one particle's 3^D contributions: shared-memory atomics when its stencil
-// lies in the window (l = window coordinates of its base), else global atomics.
-template <class R, int D>
-__device__ __forceinline__ void p2g_scatter(const Params<R> &P, const P2GFactors<R, D> &f, const int org[3], R *sm,
-                                            R4<R> *Asim, uint32_t *flags_sim, bool &escaped)
-{
-    using Gm = Geo<D>;
-    int l[D];
-    bool inside = true;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        l[a] = f.b[a] + 2 - org[a];
-        inside = inside && l[a] >= 0 && l[a] <= Gm::W - 3;
-    }
-    escaped = !inside;
-#pragma unroll
-    for (int k = 0; k < Gm::STENCIL; ++k) {
-        const int k0 = k % 3, k1 = (k / 3) % 3, k2 = k / 9;
-        R m, mom[D];
-        p2g_node<R, D>(f, P.mass, k0, k1, k2, m, mom);
-        if (inside) {
-            const int li = win_index<D>(l, k0, k1, k2);
-            atomicAdd(&sm[li], m);
-#pragma unroll
-            for (int a = 0; a < D; ++a) atomicAdd(&sm[(a + 1) * Gm::WN + li], mom[a]);
-        } else {
-            int a3[3] = {0, 0, 0}, u[3] = {0, 0, 0};
-            const int kk[3] = {k0, k1, k2};
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                a3[a] = f.b[a] + 2 + kk[a];
-                u[a] = a3[a] / Gm::T;
-            }
-            red_add4(&Asim[lin3<D>(a3, P.G_nodes)], m, mom[0], mom[1], D == 3 ? mom[D - 1] : R(0));
-            mark_node_tile(P.flags, P.node_list, P.list_count, (flags_sim - P.flags) + lin3<D>(u, P.node_tiles));
-        }
-    }
-}
-
-// Claim the next tile of the compact list (block-uniform); -1 when done.
-__device__ __forceinline__ int next_tile(int32_t *cursor, int n_tiles, int *s_slot)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) *s_slot = atomicAdd(cursor, 1);
-    __syncthreads();
-    const int k = *s_slot;
-    return k < n_tiles ? k : -1;
-}
-
 // Per-thread asynchronous copy of one element global -> shared (cp.async), in
 // commit groups the issuing thread waits for.
 template <class R> __device__ __forceinline__ void cp_async_elem(R *dst, const R *src)
@@ -510,197 +444,7 @@ template <class R> __device__ __forceinline__ void cp_async_elem(R *dst, const R
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Walks one thread's particles of a tile: cells c = threadIdx.x, +NT, ... and
-// the slots q of each cell (cell_off ranges); next() moves to the next particle.
-// (Rotating the cell of each round across the tile's columns, which balances
-// tiles cut by the body's edge, measured slower: the warps' cells then straddle
-// two layer groups.)
-template <int TN, int NT> struct CellCursor {
-    int c, q, q1;
-    __device__ __forceinline__ void start() { c = (int)threadIdx.x - NT; q = 0; q1 = 0; }
-    __device__ __forceinline__ bool next(const int32_t *off)
-    {
-        ++q;
-        while (q >= q1) {
-            c += NT;
-            if (c >= TN) return false;
-            q = off[c];
-            q1 = off[c + 1];
-        }
-        return true;
-    }
-};
-
 template <int D> constexpr int kP2GStageComps = p2g_ncomp<D>(1);
-
-// P2G.  Blocks of NT threads claim tiles dynamically; one thread per cell.  A
-// thread walks its cells' particles (slots from the position map; within a
-// group the rank planes are contiguous and cell-ordered, so the copies of a warp
-// are coalesced) through a two-stage pipeline: the components of the particle
-// after next are copied into the thread's shared-memory slots (cp.async) while
-// the current one is summed.  It sums the contributions of the particles still
-// in their cell in registers (3^D nodes x (1 + D) values) and adds them to the
-// shared-memory window when it leaves the cell.  A particle that has left its
-// cell since the sort is scattered on its own: into the window, or straight to
-// the grid if it has also left the window.  The window is added to the grid with
-// one vector atomic per touched node.  Without REG (FP64 in 3D) every particle
-// is scattered on its own.
-template <class R, int D, bool REG, int NT, int MAT>
-__global__ void __launch_bounds__(NT, (D == 3 && REG) ? MPM_P2G_MINB : 1)
-    k_p2g(const Params<R> P, const R *__restrict__ S, const int4 *__restrict__ tiles, int32_t *__restrict__ counters,
-          const int32_t *__restrict__ posmap, const int32_t *__restrict__ cell_off, R4<R> *__restrict__ A,
-          uint32_t *__restrict__ flags, unsigned long long *__restrict__ escaped_count)
-{
-    using Gm = Geo<D>;
-    constexpr int NCM = kP2GStageComps<D>;
-    constexpr int NC = p2g_ncomp<D>(MAT);             // components this material stages
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R *sm = reinterpret_cast<R *>(smem_raw);
-    int32_t *off = reinterpret_cast<int32_t *>(sm + (D + 1) * Gm::WN);
-    R *stg = reinterpret_cast<R *>(smem_raw + p2g_stage_offset<R, D>());
-    __shared__ uint32_t tile_mask;
-    __shared__ int s_slot;
-    const int n_tiles = counters[1];
-    const int tid = threadIdx.x;
-    pdl_wait();
-    for (;;) {
-        const int k = next_tile(&counters[2], n_tiles, &s_slot);
-        if (k < 0) break;
-        const int4 t = tiles[k];
-        for (int i = tid; i < (D + 1) * Gm::WN; i += NT) sm[i] = R(0);
-        for (int c = tid; c <= Gm::TN; c += NT) off[c] = cell_off[(int64_t)k * (Gm::TN + 1) + c];
-        if (tid == 0) tile_mask = 0u;
-        __syncthreads();
-        const int sim = (int)(t.x / P.tiles_per_sim);
-        int64_t tl = t.x - (int64_t)sim * P.tiles_per_sim;
-        int org[3] = {0, 0, 0};
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            org[a] = (int)(tl % P.n_tiles[a]) * Gm::T;
-            tl /= P.n_tiles[a];
-        }
-        R4<R> *Asim = A + (int64_t)sim * P.nodes_per_sim;
-        uint32_t *fsim = flags + (int64_t)sim * P.node_tiles_per_sim;
-        const int32_t *pmap = posmap + t.y;
-        bool any_escape = false;
-
-        R *const Sv = P.save_S == nullptr ? nullptr : P.save_S + t.y;
-        auto issue = [&](int stage, int32_t pos) {
-            R *dst = stg + stage * NCM * NT + tid;
-            const R *src = S + sblock((int64_t)t.y + pos, Lay<D, MAT>::NC);
-#pragma unroll
-            for (int j = 0; j < NC; ++j) cp_async_elem(dst + j * NT, src + p2g_comp<D, MAT>(j) * kPB);
-        };
-        // producer: MPM_P2G_STAGES particles ahead of the consumer, its next slot's position prefetched
-        CellCursor<Gm::TN, NT> pc, cc;
-        pc.start();
-        cc.start();
-        bool hp = pc.next(off);
-#pragma unroll
-        for (int s0 = 0; s0 < MPM_P2G_STAGES; ++s0) {
-            if (hp) issue(s0, pmap[pc.q]);
-            cp_async_commit();
-            hp = hp && pc.next(off);
-        }
-        int32_t ppos = hp ? pmap[pc.q] : 0;
-
-        bool hc = cc.next(off);
-        int stage = 0;
-        int cur = -1;                                  // cell whose accumulators are live
-        int lc[D], bown[D];
-        R acc[Gm::STENCIL][D + 1];
-        while (hc) {
-            if (cc.c != cur) {
-                cur = cc.c;
-                int r = cur;
-#pragma unroll
-                for (int a = 0; a < D; ++a) {
-                    const int ci = r % Gm::T;
-                    r /= Gm::T;
-                    lc[a] = ci + 1;                    // window coordinates of the cell's base
-                    bown[a] = org[a] + ci - 1;         // base cell index of the cell
-                }
-                if constexpr (REG) {
-#pragma unroll
-                    for (int kk = 0; kk < Gm::STENCIL; ++kk)
-#pragma unroll
-                        for (int v = 0; v <= D; ++v) acc[kk][v] = R(0);
-                }
-            }
-            cp_async_wait<MPM_P2G_STAGES - 1>();
-            P2GFactors<R, D> f;
-            {
-                const R *src = stg + stage * NCM * NT + tid;
-                if (Sv != nullptr) {                   // the adjoint's copy of this step's state
-                    R *d = Sv + pmap[cc.q];
-#pragma unroll
-                    for (int j = 0; j < NC; ++j) d[j * P.n] = src[j * NT];
-                }
-                p2g_factors<R, D, MAT>(P, [&](int j) { return src[j * NT]; }, f);
-            }
-            if (hp) issue(stage, ppos);
-            cp_async_commit();
-            hp = hp && pc.next(off);
-            if (hp) ppos = pmap[pc.q];
-            bool own = REG;
-#pragma unroll
-            for (int a = 0; a < D; ++a) own = own && (f.b[a] == bown[a]);
-            if (own) {
-                if constexpr (REG) p2g_accumulate<R, D>(f, P.mass, acc);
-            } else {
-                bool esc = false;
-                p2g_scatter<R, D>(P, f, org, sm, Asim, fsim, esc);
-                any_escape |= esc;
-            }
-            stage = stage + 1 == MPM_P2G_STAGES ? 0 : stage + 1;
-            hc = cc.next(off);
-            if constexpr (REG) {
-                if (!hc || cc.c != cur) {
-#pragma unroll
-                    for (int kk = 0; kk < Gm::STENCIL; ++kk) {
-                        const int li = win_index<D>(lc, kk % 3, (kk / 3) % 3, kk / 9);
-#pragma unroll
-                        for (int v = 0; v <= D; ++v) atomicAdd(&sm[v * Gm::WN + li], acc[kk][v]);
-                    }
-                }
-            }
-        }
-        cp_async_wait<0>();
-        const unsigned ball = __ballot_sync(0xffffffffu, any_escape);
-        if (ball && (threadIdx.x & 31) == 0) atomicAdd(escaped_count, (unsigned long long)__popc(ball));
-        __syncthreads();
-        for (int i = threadIdx.x; i < Gm::WN; i += NT) {
-            const R m = sm[i];
-            const R q0 = sm[Gm::WN + i], q1 = sm[2 * Gm::WN + i];
-            const R q2 = D == 3 ? sm[3 * Gm::WN + i] : R(0);
-            if (m != R(0) || q0 != R(0) || q1 != R(0) || q2 != R(0)) {
-                int l[3] = {0, 0, 0}, a3[3] = {0, 0, 0};
-                int r = i;
-#pragma unroll
-                for (int a = 0; a < D; ++a) {
-                    l[a] = r % Gm::W;
-                    r /= Gm::W;
-                    a3[a] = org[a] + l[a];
-                }
-                red_add4(&Asim[lin3<D>(a3, P.G_nodes)], m, q0, q1, q2);
-                unsigned bit = 0;
-#pragma unroll
-                for (int a = 0; a < D; ++a) bit |= (l[a] >= Gm::T ? 1u : 0u) << a;
-                atomicOr(&tile_mask, 1u << bit);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < (1 << D) && ((tile_mask >> threadIdx.x) & 1u)) {
-            int u[3] = {0, 0, 0};
-#pragma unroll
-            for (int a = 0; a < D; ++a) u[a] = org[a] / Gm::T + ((threadIdx.x >> a) & 1);
-            mark_node_tile(flags, P.node_list, P.list_count,
-                           (int64_t)sim * P.node_tiles_per_sim + lin3<D>(u, P.node_tiles));
-        }
-    }
-    pdl_release();
-    if (threadIdx.x == 0) counters[3] = 0;         // G2P cursor for the next kernel (G2P follows)
-}
 
 // Where k_p2g_direct takes its particles and writes its sums.  Forward P2G (MAT
 // = 0 fluid, 1 Drucker-Prager): the state S (stride ld = npad), the current sort
@@ -814,20 +558,22 @@ __device__ __noinline__ void p2g_escape(const P2GFactors<R, D> f, R mass, R4<R> 
 // pay here: pairs of two velocity components raised the register spills of the
 // 168-register 3D kernel, pairs of the nodes k2 = 0, 1 of a column measured the
 // same, 0.1251 against 0.1251 ms on the 2.76M-particle collapse.)
-template <class R, int D> struct CellSums {
+template <class R, int D, int NT> struct CellSums {
     R acc[Geo<D>::STENCIL][D + 1];
-    __device__ __forceinline__ void zero()
-    {
-#pragma unroll
-        for (int k = 0; k < Geo<D>::STENCIL; ++k)
-#pragma unroll
-            for (int v = 0; v <= D; ++v) acc[k][v] = R(0);
-    }
-    __device__ __forceinline__ void add(const P2GFactors<R, D> &f, R mp) { p2g_accumulate<R, D>(f, mp, acc); }
-    __device__ __forceinline__ R m(int k) const { return acc[k][0]; }
-    __device__ __forceinline__ R q(int k, int a) const { return a < D ? acc[k][1 + a] : R(0); }
+    __device__ __forceinline__ explicit CellSums(R *) {}
+    __device__ __forceinline__ R &at(int k, int v) { return acc[k][v]; }
+    static constexpr int kShared = 0;            // values per thread in shared memory
 };
-
+// 3D double precision: the 108 sums would take 216 of a thread's 255 registers, so those
+// of m and q_x stay there and those of q_y and q_z live in shared memory (the thread's
+// own column); the FP64 pipe's rate leaves room for their loads and stores.
+template <int NT> struct CellSums<double, 3, NT> {
+    double acc[27][2];
+    double *const sm;
+    __device__ __forceinline__ explicit CellSums(double *s) : sm(s + threadIdx.x) {}
+    __device__ __forceinline__ double &at(int k, int v) { return v < 2 ? acc[k][v] : sm[(2 * k + v - 2) * NT]; }
+    static constexpr int kShared = 54;
+};
 
 // Components staged per particle by k_p2g_direct: P2G's inputs (MAT 0, 1), or x
 // and the 21 scatter coefficients (MAT 2).
@@ -851,13 +597,17 @@ constexpr int kDirectItemInts = 40, kDirectTile = 36;
 #define MPM_P2G3_STAGES 2
 #endif
 template <int D> __host__ __device__ constexpr int direct_stages() { return D == 3 ? MPM_P2G3_STAGES : MPM_P2G2_STAGES; }
+// Dynamic shared memory: the staging slots, the sums kept there, the work items.
+template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t p2g_direct_items_offset()
+{
+    return (size_t)(direct_stages<D>() * direct_stage_comps<D, MAT>() + CellSums<R, D, NT>::kShared) * NT * sizeof(R);
+}
 template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t p2g_direct_smem()
 {
-    return (size_t)direct_stages<D>() * direct_stage_comps<D, MAT>() * NT * sizeof(R) +
-           (size_t)(NT / 32) * 2 * kDirectItemInts * sizeof(int32_t);
+    return p2g_direct_items_offset<R, D, NT, MAT>() + (size_t)(NT / 32) * 2 * kDirectItemInts * sizeof(int32_t);
 }
 
-// P2G without a shared-memory window (register accumulation, single precision).
+// P2G by cells, without a shared-memory window of the tile.
 // A work item is 32 / G cells of a tile.  Warps take items from a global cursor and
 // never synchronise with each other: each lane walks its cell's particles (with G > 1
 // every G-th of them) through a cp.async pipeline and sums those still in their cell in
@@ -866,9 +616,6 @@ template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t 
 // cell in 3D instead of 108 shared-memory atomics plus the window pass); particles that
 // left their cell are scattered on their own.  The warp marks the node tiles its cells
 // reach.
-#ifndef MPM_P2G_DIRECT
-#define MPM_P2G_DIRECT 1
-#endif
 // One round of the exchange between the lanes of a cell: of its node sums acc[0 .. N)
 // this lane keeps the lower half (or the upper one, where its bit of the lane index is
 // set), adds its partner's to it and moves it to acc[0 .. (N + 1) / 2).  first and
@@ -962,8 +709,11 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
             r /= Gm::T;
         }
     }
-    CellSums<R, D> acc;
-    acc.zero();
+    CellSums<R, D, NT> acc(stg + ST * NCM * NT);
+#pragma unroll
+    for (int k = 0; k < Gm::STENCIL; ++k)
+#pragma unroll
+        for (int v = 0; v <= D; ++v) acc.at(k, v) = R(0);
     for (; cq < q_end; cq += G) {
         cp_async_wait<ST - 1>();
         P2GFactors<R, D> f;
@@ -988,7 +738,7 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
 #pragma unroll
         for (int a = 0; a < D; ++a) own = own && (f.b[a] == bown[a]);
         if (own) {
-            acc.add(f, mass);
+            p2g_accumulate<R, D>(f, mass, [&](int k, int v) -> R & { return acc.at(k, v); });
         } else {                                   // left its cell since the sort: on its own
             any_escape = true;
             p2g_escape<R, D>(f, mass, Asim, P.G_nodes[0], P.G_nodes[1], ADJ ? nullptr : io.flags,
@@ -1017,8 +767,9 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
             const int kk = i + k0;
             if (i >= nk) continue;
             R4<R> *node = base + (kk % 3) + ((kk / 3) % 3) * sx + (kk / 9) * sxy;
-            if constexpr (ADJ) red_add4(node, acc.q(i, 0), acc.q(i, 1), acc.q(i, 2), R(0));   // (v_bar, 0)
-            else red_add4(node, acc.m(i), acc.q(i, 0), acc.q(i, 1), acc.q(i, 2));           // (m, q)
+            const R q2 = D == 3 ? acc.at(i, D) : R(0);
+            if constexpr (ADJ) red_add4(node, acc.at(i, 1), acc.at(i, 2), q2, R(0));          // (v_bar, 0)
+            else red_add4(node, acc.at(i, 0), acc.at(i, 1), acc.at(i, 2), q2);               // (m, q)
         }
     }
     cp_async_wait<0>();
@@ -1048,17 +799,16 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
 // item ahead; the next item's offsets and tile entry are copied to shared memory while
 // the current one is summed.
 template <class R, int D, int NT, int MAT, int G>
-__global__ void __launch_bounds__(NT, D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB)
+__global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB))
     k_p2g_direct(const Params<R> P, const P2GIO<R> io, unsigned long long *__restrict__ escaped_count,
                  int32_t *__restrict__ g2p_cursor)
 {
     using Gm = Geo<D>;
-    constexpr int NCM = direct_stage_comps<D, MAT>();
     constexpr int CPI = 32 / G, ITEMS = Gm::TN / CPI;     // cells per item, items per tile
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *stg = reinterpret_cast<R *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31;
-    int32_t *const s_items = reinterpret_cast<int32_t *>(smem_raw + (size_t)direct_stages<D>() * NCM * NT * sizeof(R)) +
+    int32_t *const s_items = reinterpret_cast<int32_t *>(smem_raw + p2g_direct_items_offset<R, D, NT, MAT>()) +
                              (tid >> 5) * 2 * kDirectItemInts;
     __shared__ int s_n;                              // number of items
     if (tid == 0) s_n = *io.n_tiles * ITEMS;
@@ -2074,16 +1824,17 @@ template <class R, int D> struct Launch {
         k_permute<R><<<grid_blocks(h.n, 256, ds.num_sms), 256, 0, ds.stream>>>(
             h.ncomp, h.n, h.npad, (const R *)ds.S, (R *)ds.S2, ds.perm, ds.id, ds.id2, ds.sim, ds.sim2);
     }
-    static constexpr bool kReg = (sizeof(R) == 4) || (D == 2);
-    static constexpr int kP2GThreads = (D == 3 && kReg) ? 128 : 256;
-    static size_t p2g_smem() { return p2g_smem_bytes<R, D, kP2GThreads>(); }
     // the cell-ordered P2G with G lanes per cell
     template <int MAT, int G> static void p2g_direct_launch(const HostParams &h, DevState &ds)
     {
         auto P = make_params<R>(h, ds);
         constexpr int NT = 128;
         constexpr size_t smem = p2g_direct_smem<R, D, NT, MAT>();
-        static_assert(smem <= 48 * 1024, "k_p2g_direct shared memory above the default limit");
+        static bool attr = false;
+        if (!attr) {
+            cudaFuncSetAttribute(k_p2g_direct<R, D, NT, MAT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            attr = true;
+        }
         // persistent: as many blocks as fit on the GPU at once (3D: the launch
         // bound's MPM_P2G_MINB per SM; 2D: more, its accumulators are 27 values)
         static int per_sm = 0;
@@ -2091,7 +1842,7 @@ template <class R, int D> struct Launch {
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2g_direct<R, D, NT, MAT, G>, NT, smem) !=
                     cudaSuccess ||
                 per_sm < 1)
-                per_sm = MPM_P2G_MINB;
+                per_sm = sizeof(R) == 8 ? 2 : MPM_P2G_MINB;
         }
         const int nb = ds.num_sms * per_sm;
         // tiles in key order (claiming them largest first, as G2P does, measured slower)
@@ -2110,34 +1861,13 @@ template <class R, int D> struct Launch {
     // one instantiation per material (the staged component count is a compile-time constant)
     template <int MAT> static void p2g_launch(const HostParams &h, DevState &ds)
     {
-        if constexpr (sizeof(R) == 4 && MPM_P2G_DIRECT) {
-            if (p2g_share<D>(h.n, ds.num_sms)) p2g_direct_launch<MAT, kShareLanes<D>>(h, ds);
-            else p2g_direct_launch<MAT, 1>(h, ds);
-            return;
+        if constexpr (sizeof(R) == 4) {
+            if (p2g_share<D>(h.n, ds.num_sms)) {
+                p2g_direct_launch<MAT, kShareLanes<D>>(h, ds);
+                return;
+            }
         }
-        auto P = make_params<R>(h, ds);
-        const size_t smem = p2g_smem();
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(k_p2g<R, D, kReg, kP2GThreads, MAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-            attr = true;
-        }
-        int64_t nb = ds.max_tiles;
-        const int64_t cap = (int64_t)ds.num_sms * (kP2GThreads == 128 ? MPM_P2G_MINB : 2);
-        if (nb > cap) nb = cap;
-        if (nb < 1) nb = 1;
-        launch_after(
-            k_p2g<R, D, kReg, kP2GThreads, MAT>, (int)nb, kP2GThreads, smem, ds.stream, P, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A, ds.flags, ds.escaped);
-        if (h.transfer == 3) {                       // FLIP: the momenta without forces, for v_i^n
-            auto P2 = P;
-            P2.no_force = 1;
-            P2.save_S = nullptr;
-            cudaMemsetAsync(ds.counters + 2, 0, sizeof(int32_t), ds.stream);
-            launch_after(
-                k_p2g<R, D, kReg, kP2GThreads, MAT>, (int)nb, kP2GThreads, smem, ds.stream, P2, (const R *)ds.S, ds.tiles, ds.counters, ds.posmap, ds.cell_off, (R4<R> *)ds.A2, ds.flags,
-                ds.escaped);
-        }
+        p2g_direct_launch<MAT, 1>(h, ds);
     }
     static void p2g(const HostParams &h, DevState &ds)
     {
