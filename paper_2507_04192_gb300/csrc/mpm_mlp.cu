@@ -85,24 +85,34 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
     const int64_t n = (int64_t)rows * cols;
     pdl_enter();
     double acc = 0.0;
-    for (int j = ty; j < 32; j += 8) {
-        const int r = r0 + j, c = c0 + tx;
-        if (r >= rows || c >= cols) continue;
-        const int64_t i = (int64_t)r * cols + c;
-        float g = src[i];
+    const int c1 = c0 + tx;
+    float gs[4], ys[4], zs[4];
+    auto live = [&](int j) { return r0 + ty + 8 * j < rows && c1 < cols; };
+    auto at = [&](int j) { return (int64_t)(r0 + ty + 8 * j) * cols + c1; };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!live(j)) continue;
+        gs[j] = src[at(j)];
+        ys[j] = y[at(j)];
+        zs[j] = z[at(j)];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!live(j)) continue;
+        float g = gs[j];
         if (loss != nullptr) {
-            const float e = y[i] - g;
+            const float e = ys[j] - g;
             acc += (double)e * e;
             g = 2.0f * e / (float)n;
         }
         if (!linear) {
-            const float s = 1.0f / (1.0f + expf(-z[i]));
+            const float s = 1.0f / (1.0f + expf(-zs[j]));
             g = g * (hi - lo) * s * (1.0f - s);
         }
-        dz[i] = g;
+        dz[at(j)] = g;
         const __nv_bfloat16 h = __float2bfloat16_rn(g);
-        dzb[i] = h;
-        tile[j][tx] = h;
+        dzb[at(j)] = h;
+        tile[ty + 8 * j][tx] = h;
     }
     if (loss != nullptr) {
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -118,7 +128,8 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
 // The end of a training step over all layers, one launch (a training step was 38 small
 // launches: separate conversions, transposes, column sums on one block, activation
 // gradients, Adam and copies per layer; with those in the GEMM epilogues, k_output_grad
-// and here it is 9, and 310 -> 92 us at batch 256 on 640-256-256-32): the bias gradients db[c] =
+// and here it is 9, and 310 -> 70 us at batch 256 on 640-256-256-32; the loads of a
+// block go ahead of its stores, which the compiler may not reorder: 13 us of it before): the bias gradients db[c] =
 // sum_r dz[r][c], added in the order of the rows (blocks [0, n_bias), 32 columns each,
 // 256 rows at a time through shared memory), and with update Adam on the
 // fp32 master parameters (bias-corrected moments) with the weights' bf16 copies and
@@ -139,16 +150,13 @@ struct StepEnd {
     double *loss_out;                          // when set, receives the step's loss
 };
 
-__device__ __forceinline__ float adam(float *p, float gi, float *m, float *v, const StepEnd &s)
+// Adam on one parameter p with gradient g and moments m, v.
+__device__ __forceinline__ void adam(float &p, float g, float &m, float &v, const StepEnd &s)
 {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float mi = b1 * *m + (1.f - b1) * gi;
-    const float vi = b2 * *v + (1.f - b2) * gi * gi;
-    *m = mi;
-    *v = vi;
-    const float q = *p - s.lr * (mi / s.c1) / (sqrtf(vi / s.c2) + eps);
-    *p = q;
-    return q;
+    m = b1 * m + (1.f - b1) * g;
+    v = b2 * v + (1.f - b2) * g * g;
+    p -= s.lr * (m / s.c1) / (sqrtf(v / s.c2) + eps);
 }
 
 __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEnd s)
@@ -165,11 +173,14 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
         const int c = (blk - y.bias0) * 32 + tx;
         float sum = 0.f;
         for (int r0 = 0; r0 < s.batch; r0 += 256) {
+            float d[32];                               // all loads before the first store
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 const int r = r0 + 8 * j + ty;
-                rows[8 * j + ty][tx] = r < s.batch && c < y.rows ? y.dZ[(int64_t)r * y.rows + c] : 0.f;
+                d[j] = r < s.batch && c < y.rows ? y.dZ[(int64_t)r * y.rows + c] : 0.f;
             }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) rows[8 * j + ty][tx] = d[j];
             __syncthreads();
             if (ty == 0) {                             // the loads ahead of the chain of sums
                 const int m = min(256, s.batch - r0);
@@ -187,7 +198,7 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
         }
         if (ty == 0 && c < y.rows) {
             y.gb[c] = sum;
-            if (s.update) adam(y.b + c, sum, y.mb + c, y.vb + c, s);
+            if (s.update) adam(y.b[c], sum, y.mb[c], y.vb[c], s);
         }
         return;
     }
@@ -195,13 +206,28 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
     const StepEnd::Layer &y = s.layer[l];
     const int t = blk - y.tile0, tc = (y.cols + 31) / 32;
     const int r0 = t / tc * 32, c0 = t % tc * 32;
-    for (int j = ty; j < 32; j += 8) {
-        const int r = r0 + j, c = c0 + tx;
-        if (r >= y.rows || c >= y.cols) continue;
-        const int64_t i = (int64_t)r * y.cols + c;
-        const float q = adam(y.W + i, y.gW[i], y.mW + i, y.vW + i, s);
-        y.Wb[i] = __float2bfloat16_rn(q);
-        tile[j][tx] = q;
+    // a thread's four elements are loaded before any is stored (their latencies overlap)
+    float p[4], g[4], m[4], v[4];
+    const int c1 = c0 + tx;
+    auto live = [&](int j) { return r0 + ty + 8 * j < y.rows && c1 < y.cols; };
+    auto at = [&](int j) { return (int64_t)(r0 + ty + 8 * j) * y.cols + c1; };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!live(j)) continue;
+        p[j] = y.W[at(j)];
+        g[j] = y.gW[at(j)];
+        m[j] = y.mW[at(j)];
+        v[j] = y.vW[at(j)];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!live(j)) continue;
+        adam(p[j], g[j], m[j], v[j], s);
+        y.W[at(j)] = p[j];
+        y.mW[at(j)] = m[j];
+        y.vW[at(j)] = v[j];
+        y.Wb[at(j)] = __float2bfloat16_rn(p[j]);
+        tile[ty + 8 * j][tx] = p[j];
     }
     __syncthreads();
     for (int j = ty; j < 32; j += 8) {
@@ -213,6 +239,9 @@ __global__ void __launch_bounds__(256) k_step_end(const __grid_constant__ StepEn
 int blocks_for(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 4096); }
 
 }  // namespace
+
+// Values of the pinned buffer of a network (with the status word after them).
+constexpr size_t kHostRows = 4096;
 
 struct mpm_mlp {
     int L = 0, max_batch = 0;
@@ -228,7 +257,8 @@ struct mpm_mlp {
     std::vector<__nv_bfloat16 *> dZb, dZbT;
     float *Y = nullptr, *T = nullptr, *X0f = nullptr;
     double *loss = nullptr;
-    int32_t *status = nullptr;
+    int32_t *status = nullptr;                    // after Y's last row
+    float *host = nullptr;                        // pinned, kHostRows values: small results on their way to the caller
     int64_t step = 0;
     std::string err;
 };
@@ -291,6 +321,15 @@ int check(mpm_mlp *m)
     return MPM_OK;
 }
 
+int status_code(mpm_mlp *m, int32_t st)
+{
+    if (st & kStatusTimeout) {
+        m->err = "a bounded tensor-core wait ran out";
+        return MPM_ETIMEOUT;
+    }
+    return MPM_OK;
+}
+
 int sync_status(mpm_mlp *m)
 {
     int32_t st = 0;
@@ -300,11 +339,7 @@ int sync_status(mpm_mlp *m)
         m->err = cudaGetErrorString(e);
         return MPM_ECUDA;
     }
-    if (st & kStatusTimeout) {
-        m->err = "a bounded tensor-core wait ran out";
-        return MPM_ETIMEOUT;
-    }
-    return MPM_OK;
+    return status_code(m, st);
 }
 
 // Rows of floats at src on the device: src itself, or its copy in dev (host rows, and
@@ -447,11 +482,16 @@ int mpm_mlp_create(int n_layers, const int *widths, int max_batch, double out_lo
         if (rc == MPM_OK) rc = malloc_n(m, &m->dZb[l], (size_t)B * widths[l + 1]);
         if (rc == MPM_OK) rc = malloc_n(m, &m->dZbT[l], (size_t)B * widths[l + 1]);
     }
-    if (rc == MPM_OK) rc = malloc_n(m, &m->Y, (size_t)B * widths[L]);
+    if (rc == MPM_OK) rc = malloc_n(m, &m->Y, (size_t)B * widths[L] + 1);   // the status word after the outputs
+    if (rc == MPM_OK && cudaMallocHost((void **)&m->host, kHostRows * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        m->err = "cudaMallocHost failed";
+        rc = MPM_ENOMEM;
+    }
     if (rc == MPM_OK) rc = malloc_n(m, &m->T, (size_t)B * widths[L]);
     if (rc == MPM_OK) rc = malloc_n(m, &m->X0f, (size_t)B * widths[0]);
     if (rc == MPM_OK) rc = malloc_n(m, &m->loss, 1);
-    if (rc == MPM_OK) rc = malloc_n(m, &m->status, 1);
+    if (rc == MPM_OK) m->status = reinterpret_cast<int32_t *>(m->Y + (size_t)B * widths[L]);
     if (rc == MPM_OK && cudaMemsetAsync(m->status, 0, sizeof(int32_t), m->stream) != cudaSuccess) rc = MPM_ECUDA;
     if (rc != MPM_OK) {
         mpm_mlp_destroy(m);
@@ -471,8 +511,9 @@ void mpm_mlp_destroy(mpm_mlp *m)
     for (auto *vec : {&m->Wb, &m->WbT, &m->X, &m->XT, &m->dZb, &m->dZbT})
         for (__nv_bfloat16 *p : *vec)
             if (p) cudaFree(p);
-    for (void *p : {(void *)m->Y, (void *)m->T, (void *)m->X0f, (void *)m->loss, (void *)m->status})
+    for (void *p : {(void *)m->Y, (void *)m->T, (void *)m->X0f, (void *)m->loss})
         if (p) cudaFree(p);
+    if (m->host) cudaFreeHost(m->host);
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     delete m;
 }
@@ -533,6 +574,21 @@ int mpm_mlp_infer(mpm_mlp *m, int batch, const float *x, float *y, int device_pt
     if (rc == MPM_OK) rc = check(m);
     if (rc != MPM_OK) return rc;
     const size_t n = (size_t)batch * m->w[m->L];
+    // Few outputs to the host: the rows and the status word come back in one copy through
+    // pinned memory (two pageable copies, each waited for by the driver: one row through 640-256-256-32 59 us, 49 so).
+    const size_t all = (size_t)m->max_batch * m->w[m->L] + 1;
+    if (!device_ptrs && all <= kHostRows) {
+        cudaError_t e = cudaMemcpyAsync(m->host, m->Y, sizeof(float) * all, cudaMemcpyDeviceToHost, m->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+        if (e != cudaSuccess) {
+            m->err = cudaGetErrorString(e);
+            return MPM_ECUDA;
+        }
+        int32_t st;
+        std::memcpy(&st, m->host + all - 1, sizeof st);
+        std::memcpy(y, m->host, sizeof(float) * n);
+        return status_code(m, st);
+    }
     if (cudaMemcpyAsync(y, m->Y, sizeof(float) * n, device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                         m->stream) != cudaSuccess)
         return MPM_ECUDA;
