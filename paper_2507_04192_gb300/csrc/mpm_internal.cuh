@@ -145,7 +145,7 @@ struct DevState {
     int32_t *tile_start, *tile_end;   // per tile (batch x tiles_per_sim)
     int4 *tiles;                  // compact non-empty tiles: (tile key, start, count, index) in key order
     int64_t max_tiles;
-    int4 *items;                  // G2P work items: runs of a tile's particles, largest first (same fields)
+    int4 *items;                  // G2P work items: runs of a tile's particles, largest first (k_order_items)
     int64_t max_items;
     int32_t item_q;               // particles per item, at most about (g2p_item_size)
     int32_t *perm;                // gather permutation of the last sort

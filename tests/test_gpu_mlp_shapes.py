@@ -16,7 +16,9 @@ from paper_2507_04192_gb300 import mpm
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,N,K", [(129, 33, 8), (257, 250, 264), (1280, 632, 200), (1300, 600, 72), (2560, 640, 136)])
+@pytest.mark.parametrize("M,N,K", [(129, 33, 8), (257, 250, 264), (1280, 632, 200), (1300, 600, 72), (2560, 640, 136),
+                                   # 256 columns, the last wave in two and in four parts (152 SMs)
+                                   (6390, 1000, 136), (4990, 1016, 72)])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_gemm_tile_widths(M, N, K, shift):
     g = torch.Generator().manual_seed(M + N)
