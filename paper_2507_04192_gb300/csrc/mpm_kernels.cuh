@@ -581,9 +581,8 @@ template <int D, int MAT> __host__ __device__ constexpr int direct_stage_comps()
 {
     return MAT == 2 ? 24 : kP2GStageComps<D>;
 }
-// Per warp of k_p2g_direct: two work items (the current and the next one), each its
-// cell offsets (at most 33) and, from kDirectTile on, its tile key, the tile's first
-// particle and its number.
+// Per warp of k_p2g_direct its work item: the cell offsets (at most 33) and, from
+// kDirectTile on, the tile key, the tile's first particle and the item's number.
 constexpr int kDirectItemInts = 40, kDirectTile = 36;
 // A work item of the cell-ordered P2G has 32 / G cells, G lanes for each (p2g_share): one
 // cell per lane in large problems (on the 2.76M-particle collapse P2G 0.123 ms with
@@ -604,7 +603,7 @@ template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t 
 }
 template <class R, int D, int NT, int MAT> __host__ __device__ constexpr size_t p2g_direct_smem()
 {
-    return p2g_direct_items_offset<R, D, NT, MAT>() + (size_t)(NT / 32) * 2 * kDirectItemInts * sizeof(int32_t);
+    return p2g_direct_items_offset<R, D, NT, MAT>() + (size_t)(NT / 32) * kDirectItemInts * sizeof(int32_t);
 }
 
 // P2G by cells, without a shared-memory window of the tile.
@@ -640,7 +639,7 @@ __device__ __forceinline__ void share_nodes(R (&acc)[NN][NV], int bit, int &firs
 
 // One work item: the cells [cbase, cbase + 32 / G) of a tile.  stg: this block's cp.async
 // staging slots (ST stages x NCM x NT reals); s_item: the item's offsets and tile entry in
-// shared memory; fetch_next() starts the copies of the next item's.  MAT 2 (the adjoint's
+// shared memory; fetch_next() starts the copies of the next item's over them.  MAT 2 (the adjoint's
 // v_bar scatter) is 3D only.
 template <class R, int D, int NT, int MAT, int G, class Next>
 __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<R> &io, R *stg,
@@ -691,7 +690,6 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
     const int ci0 = lane % CPI, q_end = s_item[ci0 + 1];
     const bool any = s_item[ci0] < q_end;         // the lane's cell has particles
     int pq = s_item[ci0] + lane / CPI, cq = pq;   // slots of the copies and of the sums
-    fetch_next();
 #pragma unroll
     for (int s0 = 0; s0 < ST; ++s0) {
         if (pq < q_end) issue(s0, pmap[pq]);
@@ -747,13 +745,15 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
         }
         stage = stage + 1 == ST ? 0 : stage + 1;
     }
+    __syncwarp();
+    fetch_next();                                 // under the stores of the sums
+    cp_async_commit();
     // the lane's share of the 3^D nodes: all, or nk (at most NODES) of them from k0 on
     static_assert(G == 1 || G == 4 || G == 8, "lanes per cell");
     constexpr int H1 = (Gm::STENCIL + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2;
     constexpr int NODES = G == 1 ? Gm::STENCIL : (G == 4 ? H2 : H3);
     int k0 = 0, nk = Gm::STENCIL;
     if constexpr (G > 1) {
-        __syncwarp();
         share_nodes<Gm::STENCIL>(acc.acc, 16, k0, nk);
         share_nodes<H1>(acc.acc, 8, k0, nk);
         if constexpr (G == 8) share_nodes<H2>(acc.acc, 4, k0, nk);
@@ -797,7 +797,9 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
 #endif
 // A warp's first item is its own index, later ones come from the cursor, claimed one
 // item ahead; the next item's offsets and tile entry are copied to shared memory while
-// the current one is summed.
+// the current one's sums are stored (copied ahead of its loop into a second slot they
+// cost registers: 32 steps of 1.92M water particles 5089 -> 4984 us, of 256 batched 2D
+// dam breaks 6552 -> 6429).
 template <class R, int D, int NT, int MAT, int G>
 __global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MINB : MPM_P2G2_MINB))
     k_p2g_direct(const Params<R> P, const P2GIO<R> io, unsigned long long *__restrict__ escaped_count,
@@ -809,7 +811,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MIN
     R *stg = reinterpret_cast<R *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31;
     int32_t *const s_items = reinterpret_cast<int32_t *>(smem_raw + p2g_direct_items_offset<R, D, NT, MAT>()) +
-                             (tid >> 5) * 2 * kDirectItemInts;
+                             (tid >> 5) * kDirectItemInts;
     __shared__ int s_n;                              // number of items
     if (tid == 0) s_n = *io.n_tiles * ITEMS;
     __syncthreads();
@@ -826,28 +828,28 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MIN
         const int warps = (int)gridDim.x * (NT / 32);
         return lane == 0 && s_n > warps ? warps + atomicAdd(io.cursor, 1) : s_n;
     };
-    int slot = 0, ahead = s_n;                       // ahead (lane 0): the item after the current one
+    // s: the item's offsets and tile entry; once the lanes have read them and summed their
+    // cells, the next item's take their place
+    int32_t *const s = s_items;
+    int ahead = s_n;                                 // lane 0: the item after the current one
+    bool more = false;
     {
         const int item = blockIdx.x * (NT / 32) + (tid >> 5);
-        if (item < s_n) fetch(item, s_items);        // the sort's tables: complete before the last kernel began
+        more = item < s_n;
+        if (more) fetch(item, s);                    // the sort's tables: complete before the last kernel began
         cp_async_commit();
         pdl_enter();
-        if (item < s_n) ahead = claim();
-        else slot = -1;
         cp_async_wait<0>();
     }
     __syncwarp();
-    while (slot >= 0) {
-        const int next = __shfl_sync(0xffffffffu, ahead, 0);
-        const bool more = next < s_n;
-        const int32_t *s = s_items + slot * kDirectItemInts;
-        slot = more ? slot ^ 1 : -1;
+    while (more) {
+        ahead = claim();
         p2g_direct_item<R, D, NT, MAT, G>(
             P, io, stg, s, s[kDirectTile + 2] % ITEMS * CPI,
             [&]() {
-                if (!more) return;
-                fetch(next, s_items + slot * kDirectItemInts);
-                ahead = claim();
+                const int next = __shfl_sync(0xffffffffu, ahead, 0);
+                more = next < s_n;
+                if (more) fetch(next, s);
             },
             any_escape);
         __syncwarp();
