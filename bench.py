@@ -461,7 +461,7 @@ def secondary_measurements(stream, dev):
                   "note": "host-synchronous calls incl. host<->device copies of x, targets and loss",
                   "device_train_step_ms": tr_dev, "device_train_tflops": 3 * fl_fwd / (tr_dev * 1e-3) / 1e12,
                   "device_note": "mpm_mlp_train_step_async on resident device buffers: forward, backward, Adam "
-                                 "(about 30 launches per step at this size; launch- and latency-bound)",
+                                 "(9 launches per step at three layers; launch- and latency-bound)",
                   "gemm": gemm_measurement(stream),
                   "gemm_network_shape": gemm_measurement(stream, shape=(256, 256, 640), reps=200)}
     return out

@@ -72,7 +72,7 @@ template <> struct Geo<2> {
     static constexpr int TN = T * T;             // cells per tile
     static constexpr int CELL_BITS = 8;          // log2(TN)
     static constexpr int STENCIL = 9;
-    static constexpr int NG = 256;               // cells per group (= threads of a P2G block)
+    static constexpr int NG = 256;               // cells per group
 };
 template <> struct Geo<3> {
     static constexpr int T = 8;

@@ -3,9 +3,8 @@
 // precision by mpm_kernels_f32.cu / mpm_kernels_f64.cu.
 //
 // Step (Sec. 2.2): P2G scatters mass, APIC momentum (Appendix B) and the
-// stress force of Eq. semi into a shared-memory window of the grid per tile of
-// sorted particles, then adds the window to the global grid with one vector
-// atomic per touched node; the grid update turns node momentum into velocity
+// stress force of Eq. semi, summed per cell of the sorted particles, to the grid
+// with one vector atomic per cell and node; the grid update turns node momentum into velocity
 // with gravity and the wall contact of Eq. coulomb_friction; G2P gathers the
 // node velocities back to the particles and applies the velocity gradient of
 // Eq. update_v_gradient to position, deformation gradient, density and stress.

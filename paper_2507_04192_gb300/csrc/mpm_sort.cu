@@ -1,12 +1,12 @@
 // Sorting particles by (simulation, tile, cell) and building the tile work
 // lists.  The paper scatters unsorted particles (Sec. 3.3.1, indexed
-// scatter-add); sorting is what lets P2G reduce into shared memory.
+// scatter-add); sorting is what lets P2G sum a cell's particles before it scatters.
 //
 // Keys are sorted with a stable least-significant-digit radix sort of 8-bit
 // digits: a per-block digit histogram, one exclusive scan over
 // [digit][block], and a stable scatter in which each warp ranks its elements
 // with __match_any_sync.  The sorted order then yields, per tile, its particle
-// range, which is cut into work chunks of at most `chunk` particles.
+// range, which is cut into G2P's work items.
 #include <cstdint>
 
 #include "mpm_internal.cuh"
