@@ -523,6 +523,16 @@ __device__ __forceinline__ void adj_node(const AdjStencil<R, D> &s, const int kk
     }
 }
 
+// The end of a reverse kernel lets the next one start.  In single precision the end of
+// its blocks does: an explicit release after the particle loop cost the loop registers
+// (P2G adjoint in 3D 124 -> 372 bytes of spills, launched alone on 1.36M particles 184 us,
+// 142 without; an evaluation of 40 steps 26.1 -> 23.7 ms).  In double precision the
+// earlier start is worth more (20 steps of 401,920 particles 85.2 ms with it, 85.7 without).
+template <class R> __device__ __forceinline__ void adj_release()
+{
+    if constexpr (sizeof(R) == 8) pdl_release();
+}
+
 // Adjoint of G2P for one particle: lam_in is the adjoint of S^{t+1}; writes the
 // G2P part of the adjoint of x and rho to lam_out and scatters v_bar to GVB.
 template <class R, int D>
@@ -662,7 +672,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
         for (int a = 0; a < D; ++a) lam_out[a * n + p] = xb[a];
         lam_out[JR * n + p] = rhob;
     }
-    pdl_release();
+    adj_release<R>();
 }
 
 // Adjoint of the grid update per node: GVB (adjoint of v) -> GAB (adjoint of m, P)
@@ -726,7 +736,7 @@ __global__ void __launch_bounds__(256) k_adj_grid_bwd(const Params<R> P, const R
         GAB[i] = R4<R>{mb, ob[0] * inv_m, ob[1] * inv_m, D == 3 ? ob[2] * inv_m : R(0)};
     }
     }
-    pdl_release();
+    adj_release<R>();
 }
 
 // Adjoint of P2G for one particle; completes lam_out (adjoint of S^t).
@@ -869,7 +879,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ_MINB : 1) k_adj_
         for (int q = 0; q < D * D; ++q) lam_out[(JC + q) * n + p] = Cb[q];
         lam_out[JR * n + p] += sb * dsdrho;
     }
-    pdl_release();
+    adj_release<R>();
 }
 
 // ------------------------------------------------------------------ 3D reverse kernels in separable form
@@ -1149,10 +1159,12 @@ __device__ __forceinline__ int hidx3(int b, int a)
 
 // Starts the copies into L2 of the rows a warp's next particle block (slots p0 .. p0 + 31)
 // reads in the 3D reverse particle kernels: one row per lane (a component's row starts
-// anywhere, so the lines of its first and its last element), the state's x, rho, sigma
-// and all of lam_in for the G2P adjoint, all of the state and lam_out's x, rho, sigma
-// for the P2G adjoint.  The loads follow the moments, whose registers leave no room to
-// issue them ahead (P2G adjoint 223 -> 184 us, G2P adjoint 165 -> 143 us on the 1.36M-particle problem).
+// anywhere, so the lines of its first and its last element), all of the state and
+// lam_out's x, rho, sigma for the P2G adjoint, the state's x, rho, sigma and all of
+// lam_in for the G2P adjoint.  The loads follow the moments, whose registers leave no
+// room to issue them ahead: an evaluation of 20 steps of 1.36M particles 14.42 ms without,
+// 13.65 with the P2G adjoint's; the G2P adjoint's only in double precision, as in single
+// it spills (40 -> 136 bytes) for the same time (13.69).
 template <bool G2P, class R>
 __device__ __forceinline__ void adj_prefetch(const Params<R> &P, const R *st, const R *lam, int64_t p0)
 {
@@ -1181,7 +1193,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3_MINB : 1)
     pdl_wait();
     const R cscale = R(4) * P.inv_dx;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        adj_prefetch<true, R>(P, st, lam_in, p - (threadIdx.x & 31) + (int64_t)gridDim.x * blockDim.x);
+        if constexpr (sizeof(R) == 8)
+            adj_prefetch<true, R>(P, st, lam_in, p - (threadIdx.x & 31) + (int64_t)gridDim.x * blockDim.x);
         R x[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) x[a] = st[a * n + p];
@@ -1296,7 +1309,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3_MINB : 1)
         for (int a = 0; a < D; ++a) lam_out[a * n + p] = xb[a];
         lam_out[JR * n + p] = rb1 / den;
     }
-    pdl_release();
+    adj_release<R>();
 }
 
 // 3D adjoint of P2G (same outputs as k_adj_p2g_bwd) from stencil moments of the
@@ -1402,7 +1415,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? MPM_ADJ3P_MINB : 1)
             lam_out[JR * n + p] += sb * dsdrho;
         }
     }
-    pdl_release();
+    adj_release<R>();
 }
 
 // ------------------------------------------------------------------ launchers

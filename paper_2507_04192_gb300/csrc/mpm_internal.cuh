@@ -257,7 +257,8 @@ extern const AdjOps adj_ops_f64;
 // at its end: early blocks fill whichever SM is free first, several on one, where a
 // launch onto an empty chip spreads them (32 steps of 50,560 sand particles 979 us with
 // all kernels of the step releasing early, 830 with the grid update and G2P releasing
-// late; without this launch mode adjoint evaluations of 32,768 2D and 50,560 3D particles 5.35 and 5.98 ms, 3.85 and 5.04 with it).
+// late; without this launch mode adjoint evaluations of 32,768 2D and 50,560 3D particles
+// 5.35 and 5.98 ms, 3.88 and 4.80 with it).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter()
