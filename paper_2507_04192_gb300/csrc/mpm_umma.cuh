@@ -610,6 +610,10 @@ inline cudaError_t umma_launch(const UmmaGemm *g, int n, int32_t *status, cudaSt
 // epilogue, erff on every value, and its operand stream are then spread over more
 // SMs; the deeper ring covers the L2 latency of the short tiles: one row through
 // 640-256-256-32 with its copies 84 -> 60 us, its first GEMM alone was 17 us on two SMs).
+// Up to 32 columns in more tiles than SMs: a ring of 4 stages, so that two CTAs share an SM
+// and one's loads run under the other's start and epilogue (us with 8 | 4 stages, N = 24:
+// 153 tiles, K = 640: 11.96 | 7.05, 512 tiles: 26.30 | 19.28, K = 2048: 55.84 | 47.22;
+// 152 tiles, one wave: K = 640: 7.36 | 7.15, K = 2048: 16.47 | 17.18).
 inline cudaError_t umma_gemm_tiles(const UmmaGemm *g, int n, int32_t *status, cudaStream_t stream)
 {
     int64_t tiles = 0;
@@ -619,6 +623,7 @@ inline cudaError_t umma_gemm_tiles(const UmmaGemm *g, int n, int32_t *status, cu
         widest = g[i].N > widest ? g[i].N : widest;
     }
     const int sms = umma_num_sms();
+    if (widest <= 32 && tiles > sms) return umma_launch<32, 4>(g, n, status, stream);
     if (widest <= 32 || 4 * tiles <= sms) return umma_launch<32, 8>(g, n, status, stream);
     if (2 * tiles <= sms) return umma_launch<64, 8>(g, n, status, stream);
     return umma_launch<128, MPM_UMMA_STAGES>(g, n, status, stream);
