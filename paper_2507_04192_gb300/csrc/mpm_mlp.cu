@@ -355,8 +355,9 @@ const float *on_device(mpm_mlp *m, const float *src, float *dev, int64_t n, bool
 
 // Back-propagation from the output layer's pre-activation gradient (dZ[L - 1] with its
 // bf16 forms) and, with update, one Adam step; loss_out: device copy of the loss.
-// Per layer one launch computes dW = dZ^T X and, for l > 0, dA = dZ W, whose epilogue
-// forms the layer below's dZ; then one launch ends the step.
+// Per layer one launch (two where a product fills the chip by itself) computes dW = dZ^T X
+// and, for l > 0, dA = dZ W, whose epilogue forms the layer below's dZ; then one launch
+// ends the step.
 int backward_update(mpm_mlp *m, int B, double lr, int update, double *loss_out)
 {
     const int L = m->L;
@@ -372,7 +373,7 @@ int backward_update(mpm_mlp *m, int B, double lr, int update, double *loss_out)
             epi.xnextT = m->dZbT[l - 1];
             g[1] = UmmaGemm{B, K, N, m->dZb[l], N, m->WbT[l], N, m->dZ[l - 1], K, epi};
         }
-        if (umma_gemm_tiles(g, l > 0 ? 2 : 1, m->status, m->stream) != cudaSuccess) return MPM_ECUDA;
+        if (umma_gemms(g, l > 0 ? 2 : 1, m->status, m->stream) != cudaSuccess) return MPM_ECUDA;
     }
     if (update) m->step++;
     StepEnd s{};

@@ -562,6 +562,15 @@ inline int umma_num_sms()
     return sms;
 }
 
+// Tiles of 128 x nt of an M x N product.
+inline int64_t umma_tiles(int M, int N, int nt)
+{
+    return (int64_t)((M + kUmmaM - 1) / kUmmaM) * ((N + nt - 1) / nt);
+}
+
+// Whether the 128 x 256 tiles of a product alone fill every SM: the persistent kernel's range.
+inline bool umma_wide(int M, int N, int sms) { return N >= 256 && umma_tiles(M, N, 256) >= sms; }
+
 // One GEMM C = A B^T of umma_gemm_tiles.
 struct UmmaGemm {
     int M, N, K;
@@ -619,7 +628,7 @@ inline cudaError_t umma_gemm_tiles(const UmmaGemm *g, int n, int32_t *status, cu
     int64_t tiles = 0;
     int widest = 0;
     for (int i = 0; i < n; ++i) {
-        tiles += (int64_t)((g[i].M + kUmmaM - 1) / kUmmaM) * ((g[i].N + 127) / 128);
+        tiles += umma_tiles(g[i].M, g[i].N, 128);
         widest = g[i].N > widest ? g[i].N : widest;
     }
     const int sms = umma_num_sms();
@@ -634,7 +643,7 @@ inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, in
                                  int ldb, float *C, int ldc, const UmmaEpi &epi, int32_t *status, cudaStream_t stream)
 {
     const int sms = umma_num_sms();
-    if (N >= 256 && (int64_t)((M + kUmmaM - 1) / kUmmaM) * ((N + 255) / 256) >= sms) {
+    if (umma_wide(M, N, sms)) {
         CUtensorMap tmA, tmB;
         if (!umma_tensor_map(&tmA, A, M, K, lda, kUmmaM) || !umma_tensor_map(&tmB, B, N, K, ldb, 256))
             return cudaErrorInvalidValue;
@@ -656,6 +665,37 @@ inline cudaError_t umma_gemm_tma(int M, int N, int K, const __nv_bfloat16 *A, in
     }
     const UmmaGemm g{M, N, K, A, lda, B, ldb, C, ldc, epi};
     return umma_gemm_tiles(&g, 1, status, stream);
+}
+
+// Whether two products share a launch of narrow tiles, or go one after the other so that
+// a wide one (umma_wide) takes the persistent kernel.  They share it where neither is wide,
+// and where the narrow one has tiles for less than a quarter of the SMs that take longer
+// than twice the wide one, by K-chunks of a CTA with 16 for a wide tile's epilogue: the
+// weight gradient of a small layer contracts over a large batch (256 x 256 over 65,536 rows:
+// 292 us on 16 SMs) and costs nothing beside the other product.  Two training steps, one
+// launch | one after the other: 4096-4096-4096-4096 at batch 4096 4.50 | 3.61 ms, 640-4096-32
+// at 19,456 3.62 | 3.35, 8192-8192-8192 at 512 3.67 | 3.42, 768-768-768-768 at 16,384
+// 2.80 | 2.89, 640-256-256-32 at 65,536 4.42 | 4.76.
+inline bool umma_share_launch(const UmmaGemm &a, const UmmaGemm &b, int sms)
+{
+    const bool wa = umma_wide(a.M, a.N, sms), wb = umma_wide(b.M, b.N, sms);
+    if (!wa && !wb) return true;
+    if (wa && wb) return false;
+    const UmmaGemm &w = wa ? a : b, &n = wa ? b : a;
+    const int64_t waves = (umma_tiles(w.M, w.N, 256) + sms - 1) / sms;
+    return 4 * umma_tiles(n.M, n.N, 128) <= sms && n.K / kUmmaKC >= 2 * waves * (w.K / kUmmaKC + 16);
+}
+
+// One or two independent GEMMs.
+inline cudaError_t umma_gemms(const UmmaGemm *g, int n, int32_t *status, cudaStream_t stream)
+{
+    if (n == 2 && umma_share_launch(g[0], g[1], umma_num_sms())) return umma_gemm_tiles(g, 2, status, stream);
+    for (int i = 0; i < n; ++i) {
+        const cudaError_t e = umma_gemm_tma(g[i].M, g[i].N, g[i].K, g[i].A, g[i].lda, g[i].B, g[i].ldb, g[i].C,
+                                            g[i].ldc, g[i].epi, status, stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace mpm

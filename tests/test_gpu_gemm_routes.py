@@ -1,14 +1,16 @@
 """The tensor-core GEMM where its tiles begin to outnumber the SMs: outputs of at most 32
-columns take rings of 4 stages (two CTAs per SM) from there on.
+columns take rings of 4 stages (two CTAs per SM) from there on, and the backward products
+of a network whose 128 x 256 tiles fill the chip take the persistent kernel.
 
-Values: |C - A B^T| <= 2e-5 |A| |B|^T elementwise, as in the other GEMM tests.  Time: one
-tile more than SMs must not cost a second wave of tiles (the ratio is 1.6 when it does,
-1.0 when it does not).
+Values: |C - A B^T| <= 2e-5 |A| |B|^T elementwise, gradients within 2e-2 relative L2 per
+layer, as in the other tests of GEMM and network.  Time: one tile more than SMs must not
+cost a second wave of tiles (the ratio is 1.6 when it does, 1.0 when it does not).
 """
 import numpy as np
 import pytest
 import torch
 
+from oracle import mlp as omlp
 from paper_2507_04192_gb300 import mpm
 
 pytestmark = pytest.mark.gpu
@@ -71,3 +73,31 @@ def test_one_tile_more_than_sms_is_no_second_wave():
         c = torch.empty(128 * tiles, 24, device="cuda")
         times.append(median_us(lambda: gemm(a, b, c.data_ptr(), st)))
     assert times[1] <= 1.3 * times[0], times
+
+
+def tiles(M, N):
+    return -(-M // 128) * -(-N // 256)
+
+
+@pytest.mark.parametrize("widths,batch,wide", [([40, 2312, 40], 2056, (2056, 2312)),     # dA of layer 1
+                                               ([2056, 2312, 8], 264, (2312, 2056))])    # dW of layer 0
+@pytest.mark.parametrize("hidden", ["gelu", "relu"])
+def test_wide_backward_products(widths, batch, wide, hidden):
+    assert tiles(*wide) >= sms()
+    rng = np.random.default_rng(batch)
+    p = omlp.pack([(rng.standard_normal((n, k)) / np.sqrt(k), 0.1 * rng.standard_normal(n))
+                   for k, n in zip(widths, widths[1:])]).astype(np.float32)
+    x = rng.standard_normal((batch, widths[0])).astype(np.float32)
+    t = rng.uniform(0.1, 0.6, (batch, widths[-1])).astype(np.float32)
+    net = mpm.MLP(widths, batch, hidden=mpm.MPM_ACT_RELU if hidden == "relu" else mpm.MPM_ACT_GELU)
+    net.set_params(p)
+    loss = net.train_step(x, t, lr=1e-3, update=False)
+    g = net.get_params(1).astype(np.float64)
+    net.close()
+    rl, rg = omlp.loss_and_grad(p.astype(np.float64), widths, x.astype(np.float64), t.astype(np.float64), hidden=hidden)
+    assert loss == pytest.approx(rl, rel=1e-2)
+    o = 0
+    for k, n in zip(widths, widths[1:]):
+        for m in (n * k, n):
+            assert np.linalg.norm(g[o:o + m] - rg[o:o + m]) <= 2e-2 * np.linalg.norm(rg[o:o + m])
+            o += m
