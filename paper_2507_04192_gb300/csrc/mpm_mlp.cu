@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(256) k_prepare_input(const float *__restrict__
 // Gradient of the output layer's pre-activation, dz = g (hi - lo) s (1 - s) with s =
 // sigmoid(z) (dz = g for the linear output), in fp32, bf16 and transposed bf16.
 // With a loss pointer, src holds the targets, g = 2 (y - t) / n and the loss mean
-// (y - t)^2 is added up; else src holds g = dL/dy.
+// (y - t)^2 is added up, one atomic per block (one per warp: 8192 x 1024 outputs 106 us,
+// 68 so); else src holds g = dL/dy.
 __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y, const float *__restrict__ src,
                                                      const float *__restrict__ z, float *__restrict__ dz,
                                                      __nv_bfloat16 *__restrict__ dzb, __nv_bfloat16 *__restrict__ dzbT,
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
                                                      double *__restrict__ loss)
 {
     __shared__ __nv_bfloat16 tile[32][33];
+    __shared__ double part[8];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
     const int64_t n = (int64_t)rows * cols;
     pdl_enter();
@@ -116,9 +118,13 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
     }
     if (loss != nullptr) {
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (tx == 0) atomicAdd(loss, acc / (double)n);
+        if (tx == 0) part[ty] = acc;
     }
     __syncthreads();
+    if (loss != nullptr && threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) acc += part[w];
+        atomicAdd(loss, acc / (double)n);
+    }
     for (int j = ty; j < 32; j += 8) {
         const int c = c0 + j, r = r0 + tx;
         if (r < rows && c < cols) dzbT[(int64_t)c * rows + r] = tile[tx][j];
