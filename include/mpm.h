@@ -451,8 +451,12 @@ int mpm_reset_timing(mpm_ctx *ctx);
 
 /*
  * Counters (synchronises).  out[0] active tiles, out[1] work units (tiles) after the
- * last sort, out[2] particles that took the out-of-tile path since creation,
- * out[3] sorts, out[4] steps, out[5] kernel launches since creation.
+ * last sort, out[2] particles found away from their place in the sort, since creation (see
+ * below), out[3] sorts, out[4] steps, out[5] kernel launches since creation.
+ * out[2] is a measure, not a count of particles: in double precision each P2G pass adds the
+ * cells with a particle whose stencil lies outside the window of its sort tile (the tile's
+ * nodes and one cell beyond on each side); in single precision the threads that met a
+ * particle outside its sort cell, which depends on how the cells fell to threads.
  */
 int mpm_get_stats(mpm_ctx *ctx, int64_t *out, int n);
 

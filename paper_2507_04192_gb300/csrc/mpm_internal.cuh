@@ -158,7 +158,8 @@ struct DevState {
     uint32_t *flags;              // per node tile: touched since the last grid update
     int32_t *node_list;           // the touched node tiles, in the order P2G touched them
     int32_t *status;              // device status word (bit 0: non-finite state)
-    unsigned long long *escaped;  // particles that took the out-of-window path
+    unsigned long long *escaped;  // FP64: cells with a particle outside the tile's window; FP32: threads that
+                                  // met a particle outside its cell (P2G, every pass)
     double *staging;              // n x 9 doubles for host transfers
     void *A2 = nullptr, *V2 = nullptr;   // FLIP: (m, q) without forces and the pre-update grid velocity
     void *save_A = nullptr;       // when set, the grid update also copies (m, q + dt f) ...

@@ -638,12 +638,15 @@ __device__ __forceinline__ void share_nodes(R (&acc)[NN][NV], int bit, int &firs
 
 // One work item: the cells [cbase, cbase + 32 / G) of a tile.  stg: this block's cp.async
 // staging slots (ST stages x NCM x NT reals); s_item: the item's offsets and tile entry in
-// shared memory; fetch_next() starts the copies of the next item's over them.  MAT 2 (the adjoint's
-// v_bar scatter) is 3D only.
+// shared memory; fetch_next() starts the copies of the next item's over them.  escaped
+// counts the lane's cells with a particle outside the tile's window (double precision), or
+// is true once a particle has left its cell (single).  MAT 2 (the adjoint's v_bar scatter)
+// is 3D only.
+template <class R> using Escaped = std::conditional_t<sizeof(R) == 8, int, bool>;
 template <class R, int D, int NT, int MAT, int G, class Next>
 __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<R> &io, R *stg,
                                                 const int32_t *s_item, int cbase, Next fetch_next,
-                                                bool &any_escape)
+                                                Escaped<R> &escaped)
 {
     using Gm = Geo<D>;
     constexpr bool ADJ = MAT == 2;
@@ -711,6 +714,7 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
     for (int k = 0; k < Gm::STENCIL; ++k)
 #pragma unroll
         for (int v = 0; v <= D; ++v) acc.at(k, v) = R(0);
+    bool outside = false;                         // double precision: a particle has left the tile's window
     for (; cq < q_end; cq += G) {
         cp_async_wait<ST - 1>();
         P2GFactors<R, D> f;
@@ -737,13 +741,24 @@ __device__ __forceinline__ void p2g_direct_item(const Params<R> &P, const P2GIO<
         if (own) {
             p2g_accumulate<R, D>(f, mass, [&](int k, int v) -> R & { return acc.at(k, v); });
         } else {                                   // left its cell since the sort: on its own
-            any_escape = true;
+            if constexpr (sizeof(R) == 8) {
+                int r = cbase + ci0;
+#pragma unroll
+                for (int a = 0; a < D; ++a) {      // window coordinate of the base; the own cell's is ci + 1
+                    const int ci = r % Gm::T, l = f.b[a] - bown[a] + ci + 1;
+                    r /= Gm::T;
+                    outside = outside || l < 0 || l > Gm::W - 3;
+                }
+            } else {
+                escaped = true;
+            }
             p2g_escape<R, D>(f, mass, Asim, P.G_nodes[0], P.G_nodes[1], ADJ ? nullptr : io.flags,
                              (int64_t)sim * P.node_tiles_per_sim, P.node_list, P.list_count, P.node_tiles[0],
                              P.node_tiles[1]);
         }
         stage = stage + 1 == ST ? 0 : stage + 1;
     }
+    if constexpr (sizeof(R) == 8) escaped += outside ? 1 : 0;
     __syncwarp();
     fetch_next();                                 // under the stores of the sums
     cp_async_commit();
@@ -814,7 +829,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MIN
     __shared__ int s_n;                              // number of items
     if (tid == 0) s_n = *io.n_tiles * ITEMS;
     __syncthreads();
-    bool any_escape = false;
+    Escaped<R> escaped{};
     auto fetch = [&](int item, int32_t *s) {         // copies started here, complete after a wait for all groups
         const int k = item / ITEMS;
         const int32_t *goff = io.cell_off + (int64_t)k * (Gm::TN + 1) + (item - k * ITEMS) * CPI;
@@ -850,12 +865,14 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 8 ? 2 : (D == 3 ? MPM_P2G_MIN
                 more = next < s_n;
                 if (more) fetch(next, s);
             },
-            any_escape);
+            escaped);
         __syncwarp();
     }
     if (escaped_count != nullptr) {
-        const unsigned ball = __ballot_sync(0xffffffffu, any_escape);
-        if (ball && lane == 0) atomicAdd(escaped_count, (unsigned long long)__popc(ball));
+        int sum = 0;
+        if constexpr (sizeof(R) == 8) sum = __reduce_add_sync(0xffffffffu, escaped);
+        else sum = __popc(__ballot_sync(0xffffffffu, escaped));
+        if (sum != 0 && lane == 0) atomicAdd(escaped_count, (unsigned long long)sum);
     }
     if (g2p_cursor != nullptr && threadIdx.x == 0) *g2p_cursor = 0;   // G2P cursor for the next kernel
 }

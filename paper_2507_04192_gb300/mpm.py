@@ -262,6 +262,8 @@ def mpm_reset_timing(ctx):
 
 
 def mpm_get_stats(ctx) -> dict:
+    """Counters of the context; "escaped" measures particles away from their place in the
+    sort (FP64: cells with one outside the tile's window, FP32: threads that met one outside its cell)."""
     out = (C.c_int64 * 6)()
     _check(ctx, load_library().mpm_get_stats(ctx, out, 6))
     keys = ("active_tiles", "chunks", "escaped", "sorts", "steps", "launches")
