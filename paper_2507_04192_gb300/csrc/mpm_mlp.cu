@@ -348,15 +348,38 @@ int sync_status(mpm_mlp *m)
     return status_code(m, st);
 }
 
-// Rows of floats at src on the device: src itself, or its copy in dev (host rows, and
+// Whether kernels may use a caller's device pointer in place: aligned, and memory that this
+// device knows (its own, managed or pinned).  Any other pointer is left to a copy, which
+// answers for it with an error where a kernel would fault.
+bool in_place(const void *p, size_t align)
+{
+    if (reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+    cudaPointerAttributes a{};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type != cudaMemoryTypeUnregistered && (a.type != cudaMemoryTypeDevice || a.device == dev);
+}
+
+// Copies rows of floats at src to dev (a device buffer).
+const float *copied(mpm_mlp *m, const float *src, float *dev, int64_t n, bool device)
+{
+    const cudaError_t e = cudaMemcpyAsync(dev, src, sizeof(float) * n,
+                                          device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream);
+    if (e == cudaSuccess) return dev;
+    cudaGetLastError();                           // reported by this call, not by the next one
+    m->err = cudaGetErrorString(e);
+    return nullptr;
+}
+
+// Network inputs at src on the device: src itself, or its copy in dev (host rows, and
 // device rows that kernels cannot read in place).
 const float *on_device(mpm_mlp *m, const float *src, float *dev, int64_t n, bool device)
 {
     if (device && (reinterpret_cast<uintptr_t>(src) & 3) == 0) return src;
-    if (cudaMemcpyAsync(dev, src, sizeof(float) * n, device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        m->stream) != cudaSuccess)
-        return nullptr;
-    return dev;
+    return copied(m, src, dev, n, device);
 }
 
 // Back-propagation from the output layer's pre-activation gradient (dZ[L - 1] with its
@@ -414,7 +437,7 @@ int train_queue(mpm_mlp *m, int B, const float *x, const float *src, double lr, 
 {
     const int L = m->L, nin = m->w[0], nout = m->w[L];
     const float *xd = on_device(m, x, m->X0f, (int64_t)B * nin, device);
-    const float *sd = on_device(m, src, m->T, (int64_t)B * nout, device);
+    const float *sd = device && in_place(src, sizeof(float)) ? src : copied(m, src, m->T, (int64_t)B * nout, device);
     if (!xd || !sd) return MPM_ECUDA;
     launch_after(k_prepare_input, dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream, xd, m->X[0], m->XT[0], B, nin, m->loss);
     int rc = forward(m, B, true);
@@ -619,7 +642,7 @@ int mpm_mlp_train_step_async(mpm_mlp *m, int batch, const float *x_dev, const fl
 {
     if (!m || !x_dev || !target_dev || batch < 8 || batch > m->max_batch || (batch % 8) || !(lr >= 0))
         return MPM_EINVAL;
-    const bool direct = (reinterpret_cast<uintptr_t>(loss_dev) & 7) == 0;     // a store of the last kernel
+    const bool direct = loss_dev == nullptr || in_place(loss_dev, sizeof(double));   // a store of the last kernel
     int rc = train_queue(m, batch, x_dev, target_dev, lr, 1, true, true, direct ? loss_dev : nullptr);
     if (rc != MPM_OK) return rc;
     if (!direct &&
