@@ -1433,7 +1433,10 @@ struct AdjDev {
 template <class R, int D> struct AdjLaunch {
     static int pblocks(const HostParams &h, const DevState &ds) { return grid_blocks(h.n, 256, ds.num_sms, 8); }
     // the 3D reverse particle kernels: the resident blocks, each prefetching its next round
-    static int rblocks(const HostParams &h, const DevState &ds) { return grid_blocks(h.n, 256, ds.num_sms, sizeof(R) == 4 ? 2 : 1); }
+    static int rblocks(const HostParams &h, const DevState &ds)
+    {
+        return grid_blocks(h.n, 256, ds.num_sms, sizeof(R) == 4 ? 2 : 1);
+    }
     static void save(const HostParams &h, DevState &ds, void *dst)
     {
         auto P = make_params<R>(h, ds);
@@ -1512,7 +1515,8 @@ template <class R, int D> struct AdjLaunch {
                                 a.cell_off, (R4<R> *)a.GVB, nullptr};
                     const int nb = ds.num_sms * MPM_P2G_MINB;
                     if (p2g_share<3>(h.n, ds.num_sms))
-                        launch_after(k_p2g_direct<R, 3, NT, 2, kShareLanes<3>>, nb, NT, smem, ds.stream, P, io, nullptr, nullptr);
+                        launch_after(k_p2g_direct<R, 3, NT, 2, kShareLanes<3>>, nb, NT, smem, ds.stream, P, io,
+                                     nullptr, nullptr);
                     else
                         launch_after(k_p2g_direct<R, 3, NT, 2, 1>, nb, NT, smem, ds.stream, P, io, nullptr, nullptr);
                 }
@@ -1521,21 +1525,19 @@ template <class R, int D> struct AdjLaunch {
                              (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB, (R *)nullptr);
             }
         } else {
-            launch_after(k_adj_g2p_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)GV,
-                                                                         (const R *)lam_in, (R *)lam_out,
-                                                                         (R4<R> *)a.GVB);
+            launch_after(k_adj_g2p_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st,
+                         (const R4<R> *)GV, (const R *)lam_in, (R *)lam_out, (R4<R> *)a.GVB);
         }
         int64_t nbg = h.node_tiles_per_sim;             // blocks stride the saved tile list
         if (nbg > (int64_t)ds.num_sms * 8) nbg = (int64_t)ds.num_sms * 8;
-        launch_after(k_adj_grid_bwd<R, D>, (unsigned)nbg, 256, 0, ds.stream, P, (const R4<R> *)GA, (R4<R> *)a.GVB,
-                                                                   (R4<R> *)a.GAB, GL, mub,
-                                                                   split ? a.cursor : nullptr);
+        launch_after(k_adj_grid_bwd<R, D>, (unsigned)nbg, 256, 0, ds.stream, P, (const R4<R> *)GA,
+                     (R4<R> *)a.GVB, (R4<R> *)a.GAB, GL, mub, split ? a.cursor : nullptr);
         if constexpr (D == 3 && MPM_ADJ_SEPARABLE)
-            launch_after(k_adj_p2g_bwd3<R>, rblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)a.GAB,
-                                                                   (R *)lam_out);
+            launch_after(k_adj_p2g_bwd3<R>, rblocks(h, ds), 256, 0, ds.stream, P, (const R *)st,
+                         (const R4<R> *)a.GAB, (R *)lam_out);
         else
-            launch_after(k_adj_p2g_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st, (const R4<R> *)a.GAB,
-                                                                         (R *)lam_out);
+            launch_after(k_adj_p2g_bwd<R, D>, pblocks(h, ds), 256, 0, ds.stream, P, (const R *)st,
+                         (const R4<R> *)a.GAB, (R *)lam_out);
     }
 };
 

@@ -1806,9 +1806,11 @@ Params<R> make_params(const HostParams &h, const DevState &ds)
 }
 
 // Whether the cell-ordered P2G gives a cell's particles kShareLanes lanes: the halving
-// exchanges pay while the cells are too few for the chip's lanes (32 steps without | with:
-// 2D, 8,192 particles 605 | 412 us, 294,912: 1480 | 1446, 589,824: 1639 | 1871; 3D, 50,560:
-// 1259 | 961, 86,592: 1372 | 1369, 169,680: 1491 | 1603).
+// exchanges pay while the cells are too few for the chip's lanes (32 steps without | with,
+// us: 2D, 8,192 particles 637 | 440, 258,048: 936 | 920, 294,912: 991 | 997, 368,640: 990 |
+// 1056; 3D water, 51,840: 743 | 674, 82,320: 892 | 880, 122,880: 993 | 1046; 3D sand, 25,984:
+// 737 | 646, 50,560: 818 | 837 or 804 | 735 and 67,232: 832 | 749 or 832 | 867, by where the
+// body lies on the tiles, 86,592: 990 | 1022).
 template <int D> constexpr int kShareLanes = D == 3 ? 4 : 8;
 template <int D> inline bool p2g_share(int64_t n, int num_sms)
 {
@@ -1850,7 +1852,8 @@ template <class R, int D> struct Launch {
         constexpr size_t smem = p2g_direct_smem<R, D, NT, MAT>();
         static bool attr = false;
         if (!attr) {
-            cudaFuncSetAttribute(k_p2g_direct<R, D, NT, MAT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaFuncSetAttribute(k_p2g_direct<R, D, NT, MAT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem);
             attr = true;
         }
         // persistent: as many blocks as fit on the GPU at once (3D: the launch
@@ -1898,14 +1901,14 @@ template <class R, int D> struct Launch {
         int64_t nb = h.batch * h.node_tiles_per_sim;        // blocks walk the touched-tile list
         if (nb > (int64_t)ds.num_sms * 8) nb = (int64_t)ds.num_sms * 8;
         launch_after(k_grid<R, D>, (unsigned)nb, 256, 0, ds.stream, P, (R4<R> *)ds.A, (R4<R> *)ds.V, ds.flags,
-                                                           (R4<R> *)ds.save_A, (R4<R> *)ds.save_V,
-                                                           ds.save_L, (R4<R> *)ds.A2, (R4<R> *)ds.V2,
-                                                           ds.node_list, ds.counters + 4);
+                     (R4<R> *)ds.save_A, (R4<R> *)ds.save_V, ds.save_L, (R4<R> *)ds.A2, (R4<R> *)ds.V2, ds.node_list,
+                     ds.counters + 4);
     }
     // the APIC transfer has its own instantiation; the others (TPIC, PIC, FLIP) share one
     template <bool GENERIC, int MAT> static void g2p_launch(const HostParams &h, DevState &ds)
     {
         auto P = make_params<R>(h, ds);
+        constexpr int NT = G2PSmem<R, D, MAT>::NT;
         const size_t smem = G2PSmem<R, D, MAT>::total;
         static bool attr = false;
         if (!attr) {
@@ -1916,8 +1919,8 @@ template <class R, int D> struct Launch {
         // per SM; 2D: three, its registers and shared memory allow it)
         static int per_sm = 0;
         if (per_sm == 0) {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<R, D, GENERIC, MAT>, G2PSmem<R, D, MAT>::NT,
-                                                              smem) != cudaSuccess ||
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g2p<R, D, GENERIC, MAT>, NT, smem) !=
+                    cudaSuccess ||
                 per_sm < 1)
                 per_sm = sizeof(R) == 4 ? MPM_G2P_MINB : 2;
         }
@@ -1925,9 +1928,8 @@ template <class R, int D> struct Launch {
         const int64_t cap = (int64_t)ds.num_sms * per_sm;
         if (nb > cap) nb = cap;
         if (nb < 1) nb = 1;
-        launch_after(
-            k_g2p<R, D, GENERIC, MAT>, (int)nb, G2PSmem<R, D, MAT>::NT, smem, ds.stream, P, ds.tmap_V, (R *)ds.S, (const R4<R> *)ds.V, ds.items, ds.counters, ds.status,
-            (const R4<R> *)ds.V2);
+        launch_after(k_g2p<R, D, GENERIC, MAT>, (int)nb, NT, smem, ds.stream, P, ds.tmap_V, (R *)ds.S,
+                     (const R4<R> *)ds.V, ds.items, ds.counters, ds.status, (const R4<R> *)ds.V2);
     }
     static void g2p(const HostParams &h, DevState &ds)
     {

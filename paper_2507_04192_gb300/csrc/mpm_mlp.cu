@@ -135,11 +135,11 @@ __global__ void __launch_bounds__(256) k_output_grad(const float *__restrict__ y
 // launches: separate conversions, transposes, column sums on one block, activation
 // gradients, Adam and copies per layer; with those in the GEMM epilogues, k_output_grad
 // and here it is 9, and 310 -> 70 us at batch 256 on 640-256-256-32; the loads of a
-// block go ahead of its stores, which the compiler may not reorder: 13 us of it before): the bias gradients db[c] =
-// sum_r dz[r][c], added in the order of the rows (blocks [0, n_bias), 32 columns each,
-// 256 rows at a time through shared memory), and with update Adam on the
-// fp32 master parameters (bias-corrected moments) with the weights' bf16 copies and
-// transposes (32 x 32 tiles of the weights).
+// block go ahead of its stores, which the compiler may not reorder: 13 us of it before):
+// the bias gradients db[c] = sum_r dz[r][c], added in the order of the rows (blocks
+// [0, n_bias), 32 columns each, 256 rows at a time through shared memory), and with
+// update Adam on the fp32 master parameters (bias-corrected moments) with the weights'
+// bf16 copies and transposes (32 x 32 tiles of the weights).
 constexpr int kMaxLayers = 8;
 struct StepEnd {
     struct Layer {
@@ -439,12 +439,13 @@ int train_queue(mpm_mlp *m, int B, const float *x, const float *src, double lr, 
     const float *xd = on_device(m, x, m->X0f, (int64_t)B * nin, device);
     const float *sd = device && in_place(src, sizeof(float)) ? src : copied(m, src, m->T, (int64_t)B * nout, device);
     if (!xd || !sd) return MPM_ECUDA;
-    launch_after(k_prepare_input, dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream, xd, m->X[0], m->XT[0], B, nin, m->loss);
+    launch_after(k_prepare_input, dim3((nin + 31) / 32, (B + 31) / 32), 256, 0, m->stream, xd, m->X[0], m->XT[0], B, nin,
+                 m->loss);
     int rc = forward(m, B, true);
     if (rc != MPM_OK) return rc;
-    launch_after(
-        k_output_grad, dim3((nout + 31) / 32, (B + 31) / 32), 256, 0, m->stream, m->Y, sd, m->Z[L - 1], m->dZ[L - 1], m->dZb[L - 1], m->dZbT[L - 1], B, nout, m->lo, m->hi,
-        m->out_act == MPM_OUT_LINEAR, with_loss ? m->loss : nullptr);
+    launch_after(k_output_grad, dim3((nout + 31) / 32, (B + 31) / 32), 256, 0, m->stream, m->Y, sd, m->Z[L - 1],
+                 m->dZ[L - 1], m->dZb[L - 1], m->dZbT[L - 1], B, nout, m->lo, m->hi, m->out_act == MPM_OUT_LINEAR,
+                 with_loss ? m->loss : nullptr);
     rc = backward_update(m, B, lr, update, loss_out);
     return rc != MPM_OK ? rc : check(m);
 }
