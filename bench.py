@@ -632,9 +632,9 @@ def bench_ours(args):
             "fp64": ({"value": value64, "unit": "particle-steps/s", "steps": steps64,
                       "ms_per_step": ms64 / steps64,
                       "bound": "fp64 alu",
-                      "ceiling_note": "ncu: the FP64 P2G and G2P keep the FP64 pipe busy on 81-87 % of their "
+                      "ceiling_note": "ncu: the FP64 P2G and G2P keep the FP64 pipe busy on 85-87 % of their "
                                       "active cycles (profiles/k_p2g_k_g2p_fp64_granular_cylinder_3d_128x128x64.md): "
-                                      "at most about 1.2x faster with the same FP64 instruction count"}
+                                      "at most about 1.15x faster with the same FP64 instruction count"}
                      if not args.no_fp64 else None),
             "kernels_ms_per_step": {k: kt[k][0] / max(1, args.steps) for k in kt},
             "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",

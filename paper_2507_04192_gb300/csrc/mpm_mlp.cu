@@ -605,8 +605,9 @@ int mpm_mlp_infer(mpm_mlp *m, int batch, const float *x, float *y, int device_pt
     if (rc == MPM_OK) rc = check(m);
     if (rc != MPM_OK) return rc;
     const size_t n = (size_t)batch * m->w[m->L];
-    // Few outputs to the host: the rows and the status word come back in one copy through
-    // pinned memory (two pageable copies, each waited for by the driver: one row through 640-256-256-32 59 us, 49 so).
+    // A network of small capacity, to the host: all its rows and the status word after them
+    // come back in one copy through pinned memory (two pageable copies, each waited for by the
+    // driver: one row through 640-256-256-32 built for 8 rows 59 us, 49 so).
     const size_t all = (size_t)m->max_batch * m->w[m->L] + 1;
     if (!device_ptrs && all <= kHostRows) {
         cudaError_t e = cudaMemcpyAsync(m->host, m->Y, sizeof(float) * all, cudaMemcpyDeviceToHost, m->stream);
